@@ -85,11 +85,11 @@ struct Phys {
 template <typename R>
 struct KConst {
   R alpha_r, alpha_b;
-  R crest_r, crest_b;      // (27/19)(1 - alpha_k): varphi_i^k = crest_k w_i for moving i
+  R crest3_r, crest3_b;    // (27/19)(1 - alpha_k)/3: varphi_i^k = crest_k w_i for moving i
   R nu_mid, nu_half;       // nu_bar = nu_mid + nu_half * phi
   R a_mid, a_half;         // alpha_bar = a_mid + a_half * phi
-  R A, beta;
-  R rate[27];
+  R A29, beta;             // (2/9) A of Eq. perturb; recolouring parameter
+  RelaxConst<R> rx;        // relaxation rates (relax_moments)
   R g[3];
   R rho_ref;
   int force_mode;
@@ -106,15 +106,15 @@ inline KConst<R> make_kconst(const Phys& P) {
   KConst<R> K;
   K.alpha_r = (R)P.alpha_r;
   K.alpha_b = (R)P.alpha_b;
-  K.crest_r = (R)(27.0 / 19.0 * (1.0 - P.alpha_r));
-  K.crest_b = (R)(27.0 / 19.0 * (1.0 - P.alpha_b));
+  K.crest3_r = (R)(9.0 / 19.0 * (1.0 - P.alpha_r));
+  K.crest3_b = (R)(9.0 / 19.0 * (1.0 - P.alpha_b));
   K.nu_mid = (R)(0.5 * (P.nu_r + P.nu_b));
   K.nu_half = (R)(0.5 * (P.nu_r - P.nu_b));
   K.a_mid = (R)(0.5 * (P.alpha_r + P.alpha_b));
   K.a_half = (R)(0.5 * (P.alpha_r - P.alpha_b));
-  K.A = (R)P.A;
+  K.A29 = (R)(2.0 / 9.0 * P.A);
   K.beta = (R)P.beta;
-  for (int j = 0; j < 27; ++j) K.rate[j] = (R)P.rate[j];
+  K.rx = make_relax<R>(P.rate);
   for (int a = 0; a < 3; ++a) K.g[a] = (R)P.g[a];
   K.rho_ref = (R)P.rho_ref;
   K.force_mode = P.force_mode;
@@ -612,20 +612,8 @@ struct Recol {
 // (R4), and it is carried out on the raw moments R_abc = sum_i cx^a cy^b cz^c f_i:
 //   f* = f + M^-1 (-K M h) + F' + Omega^(2),   h = f - f^(e) + F'/2
 // (Eq. scoll with Eqs. ketF-ketFd), M = T V3 (V3: raw moments, T: the sparse map
-// of Eq. momentSet).  Every term but f has the form w_i Q(c_i) + delta_{i,rest} E
-// with Q quadratic in c:
-//   f^(e) - F'/2:  C0 = P - 3/2 rho u^2 + 3/2 u.F,  V = 3 rho u - 3/2 F,
-//                  S = 9/2 rho u u + 9/2 nu_bar (u g + g u) - 9/4 (u F + F u)
-//                  (Eq. EES summed over k, Eq. varphi_ik, Eq. Phi: 16/4/1 / 48 * 2 = 9 w_i),
-//   F' + Omega^(2): C0 = -3 u.F - A|grad phi|,  V = 3 F,
-//                  S = 9/2 (u F + F u) + A|grad phi| n n
-//                  (Eq. ketFd; Eq. perturb with the square, R1, and B_i = w_i for
-//                  moving i, -10/27 at rest, Eq. B_i),
-// (P = sum_k rho_k crest_k, g = grad rho, n = grad phi/|grad phi|), whose raw
-// moments are closed forms; the rest-direction terms only touch R000 (mass),
-// which no step changes.  So: R(f) by one cascade, m = T (R(f) - closed) for
-// moments 5..27 (mass and momentum of h vanish), R* = R(f) + T^-1(-K m) +
-// closed(F' + Omega^(2)), and f* = V3^-1 R* by one inverse cascade.
+// of Eq. momentSet): one forward cascade, the relaxation of each parity class of raw moments with
+// the closed-form moments of f^(e) - F'/2 and F' + Omega^(2) (relax_moments), one inverse cascade.
 template <typename R>
 __device__ __forceinline__ Recol<R> collide(const KConst<R>& K, const R rho_r, const R ft[27], const R gphi[3],
                                             const R grho[3], R f[27]) {
@@ -643,40 +631,14 @@ __device__ __forceinline__ Recol<R> collide(const KConst<R>& K, const R rho_r, c
   const R phi = (rho_r - rho_b) * inv_rho;
   const R nubar = K.nu_mid + K.nu_half * phi;
   const R s_sh = rcp_(R(3) * nubar + R(0.5));
-  const R Pr = K.crest_r * rho_r + K.crest_b * rho_b;
-  const R g0 = grho[0], g1 = grho[1], g2 = grho[2];
-  const R uu = u0 * u0 + u1 * u1 + u2 * u2;
-  const R uF = u0 * F[0] + u1 * F[1] + u2 * F[2];
+  const R u[3] = {u0, u1, u2};
+  const R w[3] = {fma_(R(2) * nubar, grho[0], fma_(R(-0.5), F[0], f[1])),
+                  fma_(R(2) * nubar, grho[1], fma_(R(-0.5), F[1], f[3])),
+                  fma_(R(2) * nubar, grho[2], fma_(R(-0.5), F[2], f[9]))};
+  const R ug = u0 * grho[0] + u1 * grho[1] + u2 * grho[2];
+  const R Beq = fma_(nubar, ug, K.crest3_r * rho_r + K.crest3_b * rho_b);
 
-  // raw moments of h (mass and momentum of h vanish identically)
-  R h[27];
-#pragma unroll
-  for (int t = 0; t < 27; ++t) h[t] = f[t];
-  {
-    const R C0 = Pr - R(1.5) * rho * uu + R(1.5) * uF;
-    const R V[3] = {R(3) * rho * u0 - R(1.5) * F[0], R(3) * rho * u1 - R(1.5) * F[1], R(3) * rho * u2 - R(1.5) * F[2]};
-    const R r45 = R(4.5) * rho, n45 = R(4.5) * nubar;
-    const R S[6] = {r45 * u0 * u0 + R(2) * n45 * u0 * g0 - R(4.5) * u0 * F[0],
-                    r45 * u1 * u1 + R(2) * n45 * u1 * g1 - R(4.5) * u1 * F[1],
-                    r45 * u2 * u2 + R(2) * n45 * u2 * g2 - R(4.5) * u2 * F[2],
-                    r45 * u0 * u1 + n45 * (u0 * g1 + u1 * g0) - R(2.25) * (u0 * F[1] + u1 * F[0]),
-                    r45 * u1 * u2 + n45 * (u1 * g2 + u2 * g1) - R(2.25) * (u1 * F[2] + u2 * F[1]),
-                    r45 * u0 * u2 + n45 * (u0 * g2 + u2 * g0) - R(2.25) * (u0 * F[2] + u2 * F[0])};
-    closed_raw_add(h, R(-1), C0, V, S);
-  }
-  h[0] = R(0);
-  h[1] = R(0);
-  h[3] = R(0);
-  h[9] = R(0);
-  R m[27];
-  moment_forward(h, m);
-#pragma unroll
-  for (int j = 0; j < 4; ++j) m[j] = R(0);
-#pragma unroll
-  for (int j = 4; j < 27; ++j) m[j] = -(is_shear_moment(j) ? s_sh : K.rate[j]) * m[j];  // -K (M h)
-  moment_inverse_add(m, f);
-
-  // perturbation and recolouring scalars
+  // interface normal, perturbation and recolouring scalars
   Recol<R> out;
   const R G0 = gphi[0], G1 = gphi[1], G2 = gphi[2];
   const R gg = G0 * G0 + G1 * G1 + G2 * G2;
@@ -685,15 +647,9 @@ __device__ __forceinline__ Recol<R> collide(const KConst<R>& K, const R rho_r, c
   out.n0 = G0 * inv_gn;
   out.n1 = G1 * inv_gn;
   out.n2 = G2 * inv_gn;
-  const R Ag = K.A * gg * inv_gn;  // A |grad phi|
-  {
-    const R V[3] = {R(3) * F[0], R(3) * F[1], R(3) * F[2]};
-    const R S[6] = {R(9) * u0 * F[0] + Ag * out.n0 * out.n0, R(9) * u1 * F[1] + Ag * out.n1 * out.n1,
-                    R(9) * u2 * F[2] + Ag * out.n2 * out.n2, R(4.5) * (u0 * F[1] + u1 * F[0]) + Ag * out.n0 * out.n1,
-                    R(4.5) * (u1 * F[2] + u2 * F[1]) + Ag * out.n1 * out.n2,
-                    R(4.5) * (u0 * F[2] + u2 * F[0]) + Ag * out.n0 * out.n2};
-    closed_raw_add(f, R(1), R(-3) * uF - Ag, V, S);
-  }
+  const R m_abs = K.A29 * gg * inv_gn;  // (2/9) A |grad phi|
+  const R n[3] = {out.n0, out.n1, out.n2}, m[3] = {m_abs * out.n0, m_abs * out.n1, m_abs * out.n2};
+  relax_moments(K.rx, f, s_sh, Beq, u, w, F, m_abs, m, n);
   raw_inverse(f);  // f holds f*
 
   const R abar = K.a_mid + K.a_half * phi;
@@ -856,73 +812,74 @@ __device__ __forceinline__ void fused_node(const Geom& G, const FusedIO& io, int
 }
 
 // grad phi and grad rho at tile cell (lx, ly, lz) from the (rho, phi) halo tile:
-// grad chi = 3 sum_i w_i chi(x + c_i) c_i (the isotropic stencil of Sec. II).
-// w_i depends only on the speed class |c_i|^2: the neighbours of one class are
-// summed first (signs only), then the class weight multiplies once per component.
-template <int CLS, typename R, typename DT, int TXv = TX, int TYv = TY>
-__device__ __forceinline__ void class_gradients(const DT* tile, int lx, int ly, int lz, R gphi[3], R grho[3]) {
-  R sp[3] = {R(0), R(0), R(0)}, sr[3] = {R(0), R(0), R(0)};
-#pragma unroll
-  for (int t = 0; t < 27; ++t) {
-    if (speed2_of(t) != CLS) continue;
-    const DT v = tile[(lx + cx_of(t)) + TXv * ((ly + cy_of(t)) + TYv * (lz + cz_of(t)))];
-    if (cx_of(t) > 0) { sp[0] += (R)v.y; sr[0] += (R)v.x; }
-    if (cx_of(t) < 0) { sp[0] -= (R)v.y; sr[0] -= (R)v.x; }
-    if (cy_of(t) > 0) { sp[1] += (R)v.y; sr[1] += (R)v.x; }
-    if (cy_of(t) < 0) { sp[1] -= (R)v.y; sr[1] -= (R)v.x; }
-    if (cz_of(t) > 0) { sp[2] += (R)v.y; sr[2] += (R)v.x; }
-    if (cz_of(t) < 0) { sp[2] -= (R)v.y; sr[2] -= (R)v.x; }
+// grad chi = 3 sum_i w_i chi(x + c_i) c_i (the isotropic stencil of Sec. II), from the 13 differences
+// d_i = chi(x + c_i) - chi(x - c_i) of opposite neighbours.  w_i depends only on the speed class
+// |c_i|^2, so the differences of one class are summed first (signs only; the four corner pairs
+// share their partial sums) and each class weight multiplies once per component: 38 operations per
+// field, where adding the 26 neighbours one by one to each component they reach takes 63.
+template <typename R>
+struct GradOps {
+  __device__ __forceinline__ static R add(R a, R b) { return a + b; }
+  __device__ __forceinline__ static R sub(R a, R b) { return a - b; }
+  __device__ __forceinline__ static R mul(double w, R a) { return R(w) * a; }
+  __device__ __forceinline__ static R fma(double w, R a, R b) { return fma_(R(w), a, b); }
+};
+// FP32: a tile cell's (rho, phi) is one register pair, so both fields advance together in packed
+// FP32x2 instructions (a - b as a fused multiply-add by -1, the rounding of the subtraction)
+template <>
+struct GradOps<float2> {
+  __device__ __forceinline__ static float2 add(float2 a, float2 b) { return __fadd2_rn(a, b); }
+  __device__ __forceinline__ static float2 sub(float2 a, float2 b) {
+    return __ffma2_rn(b, make_float2(-1.f, -1.f), a);
   }
-  const R w = R(3.0 * weight_of(CLS == 1 ? tensor_index(1, 0, 0) : CLS == 2 ? tensor_index(1, 1, 0) : tensor_index(1, 1, 1)));
-#pragma unroll
-  for (int k = 0; k < 3; ++k) {
-    gphi[k] = fma_(w, sp[k], gphi[k]);
-    grho[k] = fma_(w, sr[k], grho[k]);
+  __device__ __forceinline__ static float2 mul(double w, float2 a) {
+    return __fmul2_rn(make_float2((float)w, (float)w), a);
   }
-}
-// FP32: a tile cell's (rho, phi) is one register pair, so the two sums of a component advance
-// together by one packed FP32x2 add (a fused multiply-add by -1 for a neighbour on the negative
-// side, which rounds exactly like the subtraction): the same operations in the same order as
-// the scalar sums above, half the instructions.  g[k] = (grad rho, grad phi) along axis k.
-template <int CLS, int TXv = TX, int TYv = TY>
-__device__ __forceinline__ void class_gradients2(const float2* tile, int lx, int ly, int lz, float2 g[3]) {
-  float2 s[3] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-  const float2 m1 = make_float2(-1.f, -1.f);
-#pragma unroll
-  for (int t = 0; t < 27; ++t) {
-    if (speed2_of(t) != CLS) continue;
-    const float2 v = tile[(lx + cx_of(t)) + TXv * ((ly + cy_of(t)) + TYv * (lz + cz_of(t)))];
-    if (cx_of(t) > 0) s[0] = __fadd2_rn(s[0], v);
-    if (cx_of(t) < 0) s[0] = __ffma2_rn(v, m1, s[0]);
-    if (cy_of(t) > 0) s[1] = __fadd2_rn(s[1], v);
-    if (cy_of(t) < 0) s[1] = __ffma2_rn(v, m1, s[1]);
-    if (cz_of(t) > 0) s[2] = __fadd2_rn(s[2], v);
-    if (cz_of(t) < 0) s[2] = __ffma2_rn(v, m1, s[2]);
+  __device__ __forceinline__ static float2 fma(double w, float2 a, float2 b) {
+    return __ffma2_rn(make_float2((float)w, (float)w), a, b);
   }
-  const float w = (float)(3.0 * weight_of(CLS == 1 ? tensor_index(1, 0, 0) : CLS == 2 ? tensor_index(1, 1, 0) : tensor_index(1, 1, 1)));
-  const float2 w2 = make_float2(w, w);
-#pragma unroll
-  for (int k = 0; k < 3; ++k) g[k] = __ffma2_rn(w2, s[k], g[k]);
+};
+// V: the value summed; get(x, y, z) the value at offset (x, y, z)
+template <typename V, class Get>
+__device__ __forceinline__ void pair_gradients(const Get& get, V g[3]) {
+  using O = GradOps<V>;
+  constexpr double w1 = 3.0 * weight_of(tensor_index(1, 0, 0)), w2 = 3.0 * weight_of(tensor_index(1, 1, 0)),
+                   w3 = 3.0 * weight_of(tensor_index(1, 1, 1));
+  {  // corners
+    const V a = O::sub(get(1, 1, 1), get(-1, -1, -1)), b = O::sub(get(1, 1, -1), get(-1, -1, 1));
+    const V c = O::sub(get(1, -1, 1), get(-1, 1, -1)), d = O::sub(get(1, -1, -1), get(-1, 1, 1));
+    const V ab = O::add(a, b), cd = O::add(c, d);
+    g[0] = O::mul(w3, O::add(ab, cd));
+    g[1] = O::mul(w3, O::sub(ab, cd));
+    g[2] = O::mul(w3, O::add(O::sub(a, b), O::sub(c, d)));
+  }
+  {  // edges
+    const V a = O::sub(get(1, 1, 0), get(-1, -1, 0)), b = O::sub(get(1, -1, 0), get(-1, 1, 0));
+    const V c = O::sub(get(1, 0, 1), get(-1, 0, -1)), d = O::sub(get(1, 0, -1), get(-1, 0, 1));
+    g[0] = O::fma(w2, O::add(O::add(a, b), O::add(c, d)), g[0]);
+    const V e = O::sub(get(0, 1, 1), get(0, -1, -1)), f = O::sub(get(0, 1, -1), get(0, -1, 1));
+    g[1] = O::fma(w2, O::add(O::sub(a, b), O::add(e, f)), g[1]);
+    g[2] = O::fma(w2, O::add(O::sub(c, d), O::sub(e, f)), g[2]);
+  }
+  g[0] = O::fma(w1, O::sub(get(1, 0, 0), get(-1, 0, 0)), g[0]);
+  g[1] = O::fma(w1, O::sub(get(0, 1, 0), get(0, -1, 0)), g[1]);
+  g[2] = O::fma(w1, O::sub(get(0, 0, 1), get(0, 0, -1)), g[2]);
 }
 
 template <typename R, typename DT, int TXv = TX, int TYv = TY>
 __device__ __forceinline__ void tile_gradients(const DT* tile, int lx, int ly, int lz, R gphi[3], R grho[3]) {
+  const DT* const c = tile + lx + TXv * (ly + TYv * lz);
   if constexpr (std::is_same<R, float>::value && std::is_same<DT, float2>::value) {
-    float2 g[3] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-    class_gradients2<1, TXv, TYv>(tile, lx, ly, lz, g);
-    class_gradients2<2, TXv, TYv>(tile, lx, ly, lz, g);
-    class_gradients2<3, TXv, TYv>(tile, lx, ly, lz, g);
+    float2 g[3];
+    pair_gradients<float2>([c](int x, int y, int z) { return c[x + TXv * (y + TYv * z)]; }, g);
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
       grho[k] = g[k].x;
       gphi[k] = g[k].y;
     }
   } else {
-#pragma unroll
-    for (int k = 0; k < 3; ++k) gphi[k] = grho[k] = R(0);
-    class_gradients<1, R, DT, TXv, TYv>(tile, lx, ly, lz, gphi, grho);
-    class_gradients<2, R, DT, TXv, TYv>(tile, lx, ly, lz, gphi, grho);
-    class_gradients<3, R, DT, TXv, TYv>(tile, lx, ly, lz, gphi, grho);
+    pair_gradients<R>([c](int x, int y, int z) { return (R)c[x + TXv * (y + TYv * z)].x; }, grho);
+    pair_gradients<R>([c](int x, int y, int z) { return (R)c[x + TXv * (y + TYv * z)].y; }, gphi);
   }
 }
 

@@ -10,8 +10,9 @@
 // follow from three one-dimensional 3-point transforms (one per axis,
 // raw_forward; raw_inverse undoes them).  The moments m_1..m_27 of
 // Eq. (momentSet) are sparse integer combinations of the R_abc
-// (moment_forward, M = T V3), and T has a sparse block inverse
-// (moment_inverse_add), so the kernels never hold a dense 27x27 matrix.
+// (moment_forward, M = T V3: the moment matrix the library exports and checks itself against), and
+// T^-1 K T falls into small blocks (relax_moments), so the kernels hold neither T nor a dense
+// 27x27 matrix.
 #pragma once
 #include <stdint.h>
 
@@ -135,10 +136,9 @@ __device__ __forceinline__ void tri_forward2(float& a0, float& a2, float& b0, fl
 }
 __device__ __forceinline__ void tri_inverse2(float& a0, float& a2, float& b0, float& b2, float& c0, float& c2) {
   const float2 k0 = make_float2(a0, a2), k1 = make_float2(b0, b2), k2 = make_float2(c0, c2);
-  const float2 h2 = __fmul2_rn(make_float2(0.5f, 0.5f), k2);
-  const float2 a = __ffma2_rn(make_float2(-0.5f, -0.5f), k1, h2);
-  const float2 b = __ffma2_rn(k2, make_float2(-1.f, -1.f), k0);
-  const float2 c = __ffma2_rn(make_float2(0.5f, 0.5f), k1, h2);
+  const float2 a = __ffma2_rn(k1, make_float2(-1.f, -1.f), k2);
+  const float2 b = __ffma2_rn(k2, make_float2(-2.f, -2.f), k0);
+  const float2 c = __fadd2_rn(k2, k1);
   a0 = a.x;
   a2 = a.y;
   b0 = b.x;
@@ -176,17 +176,18 @@ __host__ __device__ __forceinline__ void raw_forward(R v[27]) {
   for (int l = 0; l < 9; ++l) tri_forward(v[l], v[l + 9], v[l + 18]);  // z
 }
 
-// inverse of tri_forward: (k0, k1, k2) -> ((k2 - k1)/2, k0 - k2, (k2 + k1)/2).
+// inverse of tri_forward on moments whose orders 1 and 2 come halved (exactly, by a power of two):
+// (k0, k1/2, k2/2) -> ((k2 - k1)/2, k0 - k2, (k2 + k1)/2).
 template <typename R>
 __host__ __device__ __forceinline__ void tri_inverse(R& a, R& b, R& c) {
   const R k0 = a, k1 = b, k2 = c;
-  const R h2 = R(0.5) * k2;
-  a = fma_(R(-0.5), k1, h2);
-  b = k0 - k2;
-  c = fma_(R(0.5), k1, h2);
+  a = k2 - k1;
+  b = fma_(R(-2), k2, k0);
+  c = k2 + k1;
 }
 
-// populations from raw moments: the inverse of raw_forward (z, then y, then x).
+// populations from raw moments scaled by 1/2 per axis of non-zero order: the inverse of
+// raw_forward (z, then y, then x).
 template <typename R>
 __host__ __device__ __forceinline__ void raw_inverse(R v[27]) {
 #if defined(__CUDA_ARCH__)
@@ -257,83 +258,134 @@ __host__ __device__ __forceinline__ void moment_forward(const R r[27], R m[27]) 
   m[26] = LBMK_R(1, 1, 1);
 }
 
-// r += T^-1 y for a change y of the moments 5..27 (y[0..3] must be zero): the
-// inverse of the sparse map of moment_forward, block by block (scalars;
-// x-, y-, z-vectors; the three off-diagonal pairs; c_x c_y c_z).
+// ---------------------------------------------------------------------------
+// The MRT relaxation in raw moments.  The relaxation matrix K couples only raw moments of one
+// parity class (even / odd order in c_x, c_y, c_z), and Eq. (momentSet) is symmetric in the axes, so
+// T^-1 K T splits into small blocks with closed forms (S2, S4: sums of the three second-order and
+// of the three c_a^2 c_b^2 moments of h = f - f^(e) + F'/2; s: the shear rate of the node):
+//   d<a^2>       = -s h<a^2> + (s - s5)/3 S2
+//   d<b^2 c^2>   = -s19 h<b^2 c^2> + 2/3 (s - s19) h<a^2> + (s19 - s17)/3 S4
+//                  + (4/9 (s17 - s5) - 2/9 (s - s19)) S2                      (a, b, c distinct)
+//   d<222>       = -s18 h<222> + 2/3 (s18 - s17) S4 + (8/9 (s17 - s5) - 4/9 (s18 - s5)) S2
+//   d<a b>       = -s h<ab>,   d<a b c^2> = -s21 h<abc^2> + 2/3 (s21 - s) h<ab>
+//   d<a b^2>     = -(s11 + s24)/2 h<ab^2> - (s11 - s24)/2 h<ac^2>
+//   d<a b^2 c^2> = -s14 h<ab^2c^2> + 2/3 (s14 - s11) (h<ab^2> + h<ac^2>),   d<111> = -s27 h<111>
+// (S11 and S24 relax the sum and the difference of <ab^2> and <ac^2>).  The collided moments leave
+// scaled by 1/2 per axis of non-zero order, which raw_inverse expects: powers of two, folded into
+// the coefficients below, so the inverse transform needs no multiplications by 1/2.
 template <typename R>
-__host__ __device__ __forceinline__ void moment_inverse_add(const R y[27], R r[27]) {
-  // scalar block (moments 1, 5, 6, 7, 17, 18, 19, 20 <-> R000, R200, R020, R002, R220, R202, R022, R222)
-  const R dS2 = y[4];                                            // change of R200 + R020 + R002
-  const R dS4 = fma_(R(4.0 / 3.0), dS2, R(1.0 / 3.0) * y[16]);    // change of R220 + R202 + R022
-  const R d200 = R(1.0 / 3.0) * (y[5] + dS2);
-  const R d022 = R(1.0 / 9.0) * fma_(R(2), dS2, fma_(R(-6), d200, fma_(R(3), dS4, -y[18])));
-  const R dsum = dS4 - d022;                                      // change of R220 + R202
-  const R ddif = R(1.0 / 3.0) * fma_(R(2), y[6], y[19]);          // change of R220 - R202
-  const R e = dS2 - d200;
-  LBMK_R(2, 0, 0) += d200;
-  LBMK_R(0, 2, 0) = fma_(R(0.5), e + y[6], LBMK_R(0, 2, 0));
-  LBMK_R(0, 0, 2) = fma_(R(0.5), e - y[6], LBMK_R(0, 0, 2));
-  LBMK_R(0, 2, 2) += d022;
-  LBMK_R(2, 2, 0) = fma_(R(0.5), dsum + ddif, LBMK_R(2, 2, 0));
-  LBMK_R(2, 0, 2) = fma_(R(0.5), dsum - ddif, LBMK_R(2, 0, 2));
-  LBMK_R(2, 2, 2) = fma_(R(1.0 / 27.0), fma_(R(-12), dS2, fma_(R(18), dS4, y[17])), LBMK_R(2, 2, 2));
-  // vector blocks (moments 2/11/14/24, 3/12/15/25, 4/13/16/26)
-  const R vx = R(1.0 / 3.0) * y[10], vy = R(1.0 / 3.0) * y[11], vz = R(1.0 / 3.0) * y[12];
-  LBMK_R(1, 2, 0) = fma_(R(0.5), vx + y[23], LBMK_R(1, 2, 0));
-  LBMK_R(1, 0, 2) = fma_(R(0.5), vx - y[23], LBMK_R(1, 0, 2));
-  LBMK_R(1, 2, 2) = fma_(R(1.0 / 9.0), fma_(R(2), y[10], y[13]), LBMK_R(1, 2, 2));
-  LBMK_R(0, 1, 2) = fma_(R(0.5), vy + y[24], LBMK_R(0, 1, 2));
-  LBMK_R(2, 1, 0) = fma_(R(0.5), vy - y[24], LBMK_R(2, 1, 0));
-  LBMK_R(2, 1, 2) = fma_(R(1.0 / 9.0), fma_(R(2), y[11], y[14]), LBMK_R(2, 1, 2));
-  LBMK_R(2, 0, 1) = fma_(R(0.5), vz + y[25], LBMK_R(2, 0, 1));
-  LBMK_R(0, 2, 1) = fma_(R(0.5), vz - y[25], LBMK_R(0, 2, 1));
-  LBMK_R(2, 2, 1) = fma_(R(1.0 / 9.0), fma_(R(2), y[12], y[15]), LBMK_R(2, 2, 1));
-  // off-diagonal pairs (moments 8/21, 9/22, 10/23) and moment 27
-  LBMK_R(1, 1, 0) += y[7];
-  LBMK_R(1, 1, 2) = fma_(R(1.0 / 3.0), fma_(R(2), y[7], y[20]), LBMK_R(1, 1, 2));
-  LBMK_R(0, 1, 1) += y[8];
-  LBMK_R(2, 1, 1) = fma_(R(1.0 / 3.0), fma_(R(2), y[8], y[21]), LBMK_R(2, 1, 1));
-  LBMK_R(1, 0, 1) += y[9];
-  LBMK_R(1, 2, 1) = fma_(R(1.0 / 3.0), fma_(R(2), y[9], y[22]), LBMK_R(1, 2, 1));
-  LBMK_R(1, 1, 1) += y[26];
+struct RelaxConst {
+  R s5h;               // s5 / 6
+  R q1, q2, q4, q2s;   // <b^2 c^2>: (1 - s19)/4, s19/12, (s19 - s17)/12, (s17 - s5)/9
+  R s19_6;             // s19 / 6
+  R t1, t2, t4, tb;    // <222>: (1 - s18)/8, S2 and S4 coefficients / 8, s18/72
+  R v1, v2, vj;        // <a b^2>: (1 - (s11 + s24)/2)/4, -(s11 - s24)/8, s11/12
+  R z1, z2, zj;        // <a b^2 c^2>: (1 - s14)/8, (s14 - s11)/12, j coefficient / 8
+  R p1, pt, pk;        // <a b c^2>: (1 - s21)/8, s21/48, s21/12
+  R d1;                // <111>: (1 - s27)/8
+};
+
+// rate[j]: relaxation rate of moment j + 1 (the shear slots are not read)
+template <typename R>
+inline RelaxConst<R> make_relax(const double rate[27]) {
+  const double s5 = rate[4], s11 = rate[10], s14 = rate[13], s17 = rate[16], s18 = rate[17], s19 = rate[18],
+               s21 = rate[20], s24 = rate[23], s27 = rate[26];
+  RelaxConst<R> K;
+  K.s5h = (R)(s5 / 6.0);
+  K.q1 = (R)((1.0 - s19) / 4.0);
+  K.q2 = (R)(s19 / 12.0);
+  K.q4 = (R)((s19 - s17) / 12.0);
+  K.q2s = (R)((s17 - s5) / 9.0);
+  K.s19_6 = (R)(s19 / 6.0);
+  K.t1 = (R)((1.0 - s18) / 8.0);
+  K.t2 = (R)(((s17 - s5) * 8.0 / 9.0 - (s18 - s5) * 4.0 / 9.0) / 8.0);
+  K.t4 = (R)((s18 - s17) / 12.0);
+  K.tb = (R)(s18 / 72.0);
+  K.v1 = (R)((1.0 - 0.5 * (s11 + s24)) / 4.0);
+  K.v2 = (R)(-(s11 - s24) / 8.0);
+  K.vj = (R)(s11 / 12.0);
+  K.z1 = (R)((1.0 - s14) / 8.0);
+  K.z2 = (R)((s14 - s11) / 12.0);
+  K.zj = (R)((s14 / 9.0 - (s14 - s11) * 4.0 / 9.0) / 8.0);
+  K.p1 = (R)((1.0 - s21) / 8.0);
+  K.pt = (R)(s21 / 48.0);
+  K.pk = (R)(s21 / 12.0);
+  K.d1 = (R)((1.0 - s27) / 8.0);
+  return K;
 }
 
-// Raw moments of g_i = w_i Q(c_i), Q(c) = C0 + c.V + c.S.c with S symmetric
-// (S = {Sxx, Syy, Szz, Sxy, Syz, Sxz}): products of the D1Q3 weight moments
-// sum W(c) c^k = 1, 0, 1/3, 0, 1/3 (k = 0..4).  r_abc += sign * R_abc[g] for
-// every raw moment except R000 (whose change the caller fixes).
+// Raw moments r of the total populations -> raw moments of f* = f - M^-1 K M h + F' + Omega^(2),
+// scaled as raw_inverse expects.  Every term but f has the form w_i Q(c_i) (+ a rest-direction
+// term, which only touches the conserved mass moment) with Q quadratic in c, so its raw moments are
+// products of the D1Q3 weight moments 1, 1/3.  With w = rho u - F/2 + 2 nu_bar grad(rho) - F/2 and
+// B = (P + 3 nu_bar u.grad(rho))/3 (P: sum_k rho_k crest_k; Eqs. EES, varphi_ik, Phi), the
+// equilibrium minus half the forcing has the moments
+//   <a^2> = B + u_a w_a,  <b^2c^2> = (B + u_b w_b + u_c w_c)/3,  <222> = (B + u.w)/9,
+//   <ab> = (u_a w_b + u_b w_a)/2 = 3 <abc^2>,  <ab^2> = <ac^2> = 3 <ab^2c^2> = j_a/3
+// (j_a = <a>: the F/2 terms cancel), and F' + Omega^(2) (Eq. ketFd; Eq. perturb, B_i) with
+// pi_a = 2 u_a F_a + m_a n_a, m = (2/9) A |grad phi| n
+//   <a> = F_a,  <a^2> = pi_a - |m|,  <b^2c^2> = (sum pi - |m| - pi_a)/3,  <222> = (sum pi - |m|)/9,
+//   <ab> = u_a F_b + u_b F_a + m_a n_b = 3 <abc^2>,  <ab^2> = <ac^2> = 3 <ab^2c^2> = F_a/3.
+// About 170 operations; relaxing the 23 moments of Eq. (momentSet) one by one between T and T^-1,
+// with the closed forms added per raw moment, took about 330.  Measured with the gradients by
+// opposite pairs: collide-stream pass in FP64 on a 32^3 box (bound by the FP64 pipe) 69 -> 56 us;
+// packed half, interior tiles of a 128^3 jet (bound by instruction issue) 78 -> 72 us on even and
+// 88 -> 85 us on odd steps, 1048 -> 912 and 1210 -> 1089 instructions a node.
 template <typename R>
-__host__ __device__ __forceinline__ void closed_raw_add(R r[27], R sign, R C0, const R V[3], const R S[6]) {
-  const R t3 = R(1.0 / 3.0) * sign, t9 = R(1.0 / 9.0) * sign, t27 = R(1.0 / 27.0) * sign;
-  const R Sxx = S[0], Syy = S[1], Szz = S[2];
-  const R a = C0 + Sxx, b = C0 + Syy, c = C0 + Szz, yz = Syy + Szz, xz = Sxx + Szz, xy = Sxx + Syy;
-  LBMK_R(1, 0, 0) = fma_(t3, V[0], LBMK_R(1, 0, 0));
-  LBMK_R(0, 1, 0) = fma_(t3, V[1], LBMK_R(0, 1, 0));
-  LBMK_R(0, 0, 1) = fma_(t3, V[2], LBMK_R(0, 0, 1));
-  LBMK_R(2, 0, 0) = fma_(t3, a, fma_(t9, yz, LBMK_R(2, 0, 0)));
-  LBMK_R(0, 2, 0) = fma_(t3, b, fma_(t9, xz, LBMK_R(0, 2, 0)));
-  LBMK_R(0, 0, 2) = fma_(t3, c, fma_(t9, xy, LBMK_R(0, 0, 2)));
-  LBMK_R(2, 2, 0) = fma_(t9, a + Syy, fma_(t27, Szz, LBMK_R(2, 2, 0)));
-  LBMK_R(2, 0, 2) = fma_(t9, a + Szz, fma_(t27, Syy, LBMK_R(2, 0, 2)));
-  LBMK_R(0, 2, 2) = fma_(t9, b + Szz, fma_(t27, Sxx, LBMK_R(0, 2, 2)));
-  LBMK_R(2, 2, 2) = fma_(t27, a + yz, LBMK_R(2, 2, 2));
-  const R v0 = t9 * V[0], v1 = t9 * V[1], v2 = t9 * V[2];
-  LBMK_R(1, 2, 0) += v0;
-  LBMK_R(1, 0, 2) += v0;
-  LBMK_R(1, 2, 2) = fma_(t27, V[0], LBMK_R(1, 2, 2));
-  LBMK_R(2, 1, 0) += v1;
-  LBMK_R(0, 1, 2) += v1;
-  LBMK_R(2, 1, 2) = fma_(t27, V[1], LBMK_R(2, 1, 2));
-  LBMK_R(2, 0, 1) += v2;
-  LBMK_R(0, 2, 1) += v2;
-  LBMK_R(2, 2, 1) = fma_(t27, V[2], LBMK_R(2, 2, 1));
-  const R u9 = R(2) * t9, u27 = R(2) * t27;
-  LBMK_R(1, 1, 0) = fma_(u9, S[3], LBMK_R(1, 1, 0));
-  LBMK_R(1, 1, 2) = fma_(u27, S[3], LBMK_R(1, 1, 2));
-  LBMK_R(0, 1, 1) = fma_(u9, S[4], LBMK_R(0, 1, 1));
-  LBMK_R(2, 1, 1) = fma_(u27, S[4], LBMK_R(2, 1, 1));
-  LBMK_R(1, 0, 1) = fma_(u9, S[5], LBMK_R(1, 0, 1));
-  LBMK_R(1, 2, 1) = fma_(u27, S[5], LBMK_R(1, 2, 1));
+__host__ __device__ __forceinline__ void relax_moments(const RelaxConst<R>& K, R r[27], R s_sh, R B, const R u[3],
+                                                       const R w[3], const R F[3], R m_abs, const R m[3],
+                                                       const R n[3]) {
+  // second-order and even moments
+  const R sg0 = u[0] * w[0], sg1 = u[1] * w[1], sg2 = u[2] * w[2];
+  const R tr = sg0 + sg1 + sg2, Btr = B + tr;
+  const R pi0 = fma_(u[0], F[0], fma_(u[0], F[0], m[0] * n[0]));
+  const R pi1 = fma_(u[1], F[1], fma_(u[1], F[1], m[1] * n[1]));
+  const R pi2 = fma_(u[2], F[2], fma_(u[2], F[2], m[2] * n[2]));
+  const R Z = pi0 + pi1 + pi2 - m_abs;
+  const R h0 = LBMK_R(2, 0, 0) - B - sg0, h1 = LBMK_R(0, 2, 0) - B - sg1, h2 = LBMK_R(0, 0, 2) - B - sg2;
+  const R S2 = h0 + h1 + h2;
+  const R S4 = LBMK_R(2, 2, 0) + LBMK_R(0, 2, 2) + LBMK_R(2, 0, 2) - fma_(R(2.0 / 3.0), tr, B);
+  const R c = fma_(R(-0.5), s_sh, R(0.5));                              // (1 - s)/2
+  const R L = fma_(fma_(R(1.0 / 6.0), s_sh, -K.s5h), S2, R(0.5) * (B - m_abs));
+  LBMK_R(2, 0, 0) = fma_(c, h0, fma_(R(0.5), sg0 + pi0, L));
+  LBMK_R(0, 2, 0) = fma_(c, h1, fma_(R(0.5), sg1 + pi1, L));
+  LBMK_R(0, 0, 2) = fma_(c, h2, fma_(R(0.5), sg2 + pi2, L));
+  const R b = fma_(R(1.0 / 6.0), s_sh, -K.s19_6);                        // (s - s19)/6
+  const R a2 = fma_(R(-1.0 / 3.0), b, K.q2s);
+  const R CQ = fma_(a2, S2, fma_(K.q4, S4, fma_(R(1.0 / 12.0), Z, K.q2 * Btr)));
+  LBMK_R(0, 2, 2) = fma_(K.q1, LBMK_R(0, 2, 2), fma_(b, h0, fma_(-K.q2, sg0, fma_(R(-1.0 / 12.0), pi0, CQ))));
+  LBMK_R(2, 0, 2) = fma_(K.q1, LBMK_R(2, 0, 2), fma_(b, h1, fma_(-K.q2, sg1, fma_(R(-1.0 / 12.0), pi1, CQ))));
+  LBMK_R(2, 2, 0) = fma_(K.q1, LBMK_R(2, 2, 0), fma_(b, h2, fma_(-K.q2, sg2, fma_(R(-1.0 / 12.0), pi2, CQ))));
+  LBMK_R(2, 2, 2) =
+      fma_(K.t1, LBMK_R(2, 2, 2), fma_(K.t4, S4, fma_(K.t2, S2, fma_(K.tb, Btr, R(1.0 / 72.0) * Z))));
+  // pairs <ab>, <abc^2>
+  const R c4 = R(0.5) * c, k = fma_(R(-1.0 / 12.0), s_sh, K.pk);         // (1 - s)/4, (s21 - s)/12
+#define LBMK_PAIR(P, Q, x, y)                                                                       \
+  {                                                                                                 \
+    const R t = fma_(u[x], w[y], u[y] * w[x]);                                                      \
+    const R g = fma_(m[x], n[y], fma_(u[x], F[y], u[y] * F[x]));                                    \
+    const R h = fma_(R(-0.5), t, P);                                                                \
+    P = fma_(c4, h, fma_(R(0.125), t, R(0.25) * g));                                                \
+    Q = fma_(K.p1, Q, fma_(K.pt, t, fma_(k, h, R(1.0 / 24.0) * g)));                                \
+  }
+  LBMK_PAIR(LBMK_R(1, 1, 0), LBMK_R(1, 1, 2), 0, 1)
+  LBMK_PAIR(LBMK_R(0, 1, 1), LBMK_R(2, 1, 1), 1, 2)
+  LBMK_PAIR(LBMK_R(1, 0, 1), LBMK_R(1, 2, 1), 0, 2)
+#undef LBMK_PAIR
+  // vectors <a>, <ab^2>, <ac^2>, <ab^2c^2>
+#define LBMK_VEC(J, P, Q, T, x)                                                                     \
+  {                                                                                                 \
+    const R j = J, e = fma_(K.vj, j, R(1.0 / 12.0) * F[x]), p = P, q = Q;                            \
+    J = R(0.5) * (j + F[x]);                                                                        \
+    P = fma_(K.v1, p, fma_(K.v2, q, e));                                                            \
+    Q = fma_(K.v1, q, fma_(K.v2, p, e));                                                            \
+    T = fma_(K.z1, T, fma_(K.z2, p + q, fma_(K.zj, j, R(1.0 / 72.0) * F[x])));                       \
+  }
+  LBMK_VEC(LBMK_R(1, 0, 0), LBMK_R(1, 2, 0), LBMK_R(1, 0, 2), LBMK_R(1, 2, 2), 0)
+  LBMK_VEC(LBMK_R(0, 1, 0), LBMK_R(0, 1, 2), LBMK_R(2, 1, 0), LBMK_R(2, 1, 2), 1)
+  LBMK_VEC(LBMK_R(0, 0, 1), LBMK_R(2, 0, 1), LBMK_R(0, 2, 1), LBMK_R(2, 2, 1), 2)
+#undef LBMK_VEC
+  LBMK_R(1, 1, 1) = K.d1 * LBMK_R(1, 1, 1);
 }
 
 #undef LBMK_R
