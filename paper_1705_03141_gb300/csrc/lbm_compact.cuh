@@ -733,25 +733,18 @@ __global__ void k_init_c(CompactStore<BF16> st, Geom G, const __grid_constant__ 
   const int64_t n = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (n >= N) return;
   const int x = (int)(n % G.nx), y = (int)((n / G.nx) % G.ny), z = (int)(n / ((int64_t)G.nx * G.ny));
-  const double u0 = u ? u[n] : 0.0, u1 = u ? u[N + n] : 0.0, u2 = u ? u[2 * N + n] : 0.0;
-  const double uu = u0 * u0 + u1 * u1 + u2 * u2;
   const double r = rr[n], b = rb[n];
-  const double ar = K.alpha_r_d, ab = 8.0 / 27.0;
   const int64_t sn = snode(G, x, y, z);
-#pragma unroll
-  for (int t = 0; t < 27; ++t) {  // the lattice constants fold at compile time
-    const double w = weight_of(t);
-    const double cu = cx_of(t) * u0 + cy_of(t) * u1 + cz_of(t) * u2;
-    const double poly = w * (3.0 * cu + 4.5 * cu * cu - 1.5 * uu);
-    const double vr = t == REST ? ar : 27.0 / 19.0 * (1.0 - ar) * w;
-    const double vb = t == REST ? ab : 27.0 / 19.0 * (1.0 - ab) * w;
-    const double fr = r * (vr + poly), fb = b * (vb + poly);
-    st.store(sn, t, speed2_of(t), K, (float)(fr + fb));
-    if (on_top(G, z)) {
-      G.ctop[((int64_t)x + (int64_t)G.nx * y) * 64 + t] = (float)fr;
-      G.ctop[((int64_t)x + (int64_t)G.nx * y) * 64 + 32 + t] = (float)fb;
-    }
-  }
+  const bool top = on_top(G, z);
+  float* const tp = G.ctop + ((int64_t)x + (int64_t)G.nx * y) * 64;
+  equilibrium_pairs<DF>(r, b, u ? u[n] : 0.0, u ? u[N + n] : 0.0, u ? u[2 * N + n] : 0.0, K.alpha_r_d,
+                        [&](int t, DF fr, DF fb) {
+                          st.store(sn, t, speed2_of(t), K, narrow_(add_(fr, fb)));
+                          if (top) {
+                            tp[t] = narrow_(fr);
+                            tp[32 + t] = narrow_(fb);
+                          }
+                        });
   dens[n] = make_float2((float)(r + b), (float)((r - b) / (r + b)));
 }
 
@@ -765,38 +758,46 @@ __global__ void k_macro_c(CompactStore<BF16> st, Geom G, const __grid_constant__
   const int64_t n = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (n >= N) return;
   const int x = (int)(n % G.nx), y = (int)((n / G.nx) % G.ny), z = (int)(n / ((int64_t)G.nx * G.ny));
-  double rho = 0.0, j[3] = {0.0, 0.0, 0.0}, red = 0.0;
   const bool top = on_top(G, z);
   NodeMap nm;
   nm.init(G, x, y, z);
+  DF srho = {0.f, 0.f}, sred = {0.f, 0.f}, m[3] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
+  float f[27];
+#pragma unroll
   for (int t = 0; t < 27; ++t) {
-    double f;
     if (top) {
       const float* tp = G.ctop + ((int64_t)x + (int64_t)G.nx * y) * 64;
-      f = (double)tp[t] + (double)tp[32 + t];
-      red += (double)tp[t];
+      const DF s = two_sum(tp[t], tp[32 + t]);
+      acc_(sred, tp[t]);
+      acc_(srho, s);
+      if (cx_of(t)) acc_(m[0], cx_of(t) > 0 ? s : neg_(s));
+      if (cy_of(t)) acc_(m[1], cy_of(t) > 0 ? s : neg_(s));
+      if (cz_of(t)) acc_(m[2], cz_of(t) > 0 ? s : neg_(s));
     } else {
       int64_t node;
       int dir;
       slot_of(nm, layout, t, node, dir);
-      f = (double)st.load(node, dir, speed2_of(t), K);
+      f[t] = st.load(node, dir, speed2_of(t), K);
+      acc_(srho, f[t]);
     }
-    rho += f;
-    j[0] += cx_of(t) * f;
-    j[1] += cy_of(t) * f;
-    j[2] += cz_of(t) * f;
   }
-  if (!top) red = 0.5 * rho * (1.0 + (double)dens[n].y);
-  double k = 0.0;
-  if (K.force_mode == FORCE_BUOYANCY || K.force_mode == FORCE_DISPERSED) k = rho - (double)K.rho_ref;
-  else if (K.force_mode == FORCE_UNIFORM) k = 1.0;
-  if (rr) rr[n] = red;
-  if (rb) rb[n] = rho - red;
-  if (u) {
-    u[n] = (j[0] + 0.5 * k * (double)K.g[0]) / rho;
-    u[N + n] = (j[1] + 0.5 * k * (double)K.g[1]) / rho;
-    u[2 * N + n] = (j[2] + 0.5 * k * (double)K.g[2]) / rho;
+  if (!top && u) {
+#pragma unroll
+    for (int t = 14; t < 27; ++t) {
+      const DF d = two_sum(f[t], -f[26 - t]);
+      if (cx_of(t)) acc_(m[0], cx_of(t) > 0 ? d : neg_(d));
+      if (cy_of(t)) acc_(m[1], cy_of(t) > 0 ? d : neg_(d));
+      if (cz_of(t)) acc_(m[2], cz_of(t) > 0 ? d : neg_(d));
+    }
   }
+  if (rr || rb) {
+    const double rho = to_f64(srho);
+    double red = to_f64(sred);
+    if (!top) red = 0.5 * rho * (1.0 + (double)dens[n].y);
+    if (rr) rr[n] = red;
+    if (rb) rb[n] = rho - red;
+  }
+  if (u) write_velocity(K, srho, m, u, n, N);
 }
 
 // one direction (paper order) of the canonical FP64 arrays <- storage, colours rebuilt

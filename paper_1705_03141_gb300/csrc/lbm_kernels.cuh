@@ -30,6 +30,7 @@
 
 #include <type_traits>
 
+#include "lbm_df.cuh"
 #include "lbm_lattice.cuh"
 #include "lbm_tma.cuh"
 
@@ -1800,29 +1801,66 @@ __global__ void __launch_bounds__(256) k_outflow(Store st, Geom G,
 // ---------------------------------------------------------------------------
 // initial state / population I/O / macroscopic fields (FP64 buffers on the device)
 
+// Per-colour equilibria f^k = rho_k (varphi_i(alpha_k) + w_i (3 c.u + 9/2 (c.u)^2 - 3/2 u^2)) of Eq.
+// (EES) with Phi = 0, alpha_b = 8/27, given to put(t, f^r, f^b) in opposite pairs: the pair shares
+// its even part, the colours share the polynomial, and varphi_i = (27/19)(1 - alpha_k) w_i of the
+// moving directions leaves one multiply-add per value (about 140 operations a node; direction by
+// direction it took about 540).
+template <typename T, class Put>
+__device__ __forceinline__ void equilibrium_pairs(double rd, double bd, double u0d, double u1d, double u2d, double ar,
+                                                  const Put& put) {
+  const T r = wide_<T>(rd), b = wide_<T>(bd), u0 = wide_<T>(u0d), u1 = wide_<T>(u1d), u2 = wide_<T>(u2d);
+  const T base = mul_(wide_<T>(-1.5), mad_(u0, u0, mad_(u1, u1, mul_(u2, u2))));
+  const T vr = mul_(r, wide_<T>(27.0 / 19.0 * (1.0 - ar))), vb = mul_(b, wide_<T>(27.0 / 19.0 * (1.0 - 8.0 / 27.0)));
+  const auto pair = [&](int t, T rw, T bw, T rv, T bv, T cu) {
+    const T q = mad_(mul_(wide_<T>(4.5), cu), cu, base), c3 = mul_(wide_<T>(3.0), cu);
+    const T p = add_(q, c3), n = sub_(q, c3);
+    put(t, mad_(rw, p, rv), mad_(bw, p, bv));
+    put(26 - t, mad_(rw, n, rv), mad_(bw, n, bv));
+  };
+  {
+    const T w = wide_<T>(weight_of(REST));
+    put(REST, mad_(mul_(r, w), base, mul_(r, wide_<T>(ar))), mad_(mul_(b, w), base, mul_(b, wide_<T>(8.0 / 27.0))));
+  }
+  {
+    const T w = wide_<T>(weight_of(tensor_index(1, 0, 0)));
+    const T rw = mul_(r, w), bw = mul_(b, w), rv = mul_(vr, w), bv = mul_(vb, w);
+    pair(tensor_index(1, 0, 0), rw, bw, rv, bv, u0);
+    pair(tensor_index(0, 1, 0), rw, bw, rv, bv, u1);
+    pair(tensor_index(0, 0, 1), rw, bw, rv, bv, u2);
+  }
+  const T sxy = add_(u0, u1), dxy = sub_(u0, u1);
+  {
+    const T w = wide_<T>(weight_of(tensor_index(1, 1, 0)));
+    const T rw = mul_(r, w), bw = mul_(b, w), rv = mul_(vr, w), bv = mul_(vb, w);
+    pair(tensor_index(1, 1, 0), rw, bw, rv, bv, sxy);
+    pair(tensor_index(1, -1, 0), rw, bw, rv, bv, dxy);
+    pair(tensor_index(1, 0, 1), rw, bw, rv, bv, add_(u0, u2));
+    pair(tensor_index(1, 0, -1), rw, bw, rv, bv, sub_(u0, u2));
+    pair(tensor_index(0, 1, 1), rw, bw, rv, bv, add_(u1, u2));
+    pair(tensor_index(0, 1, -1), rw, bw, rv, bv, sub_(u1, u2));
+  }
+  const T w = wide_<T>(weight_of(tensor_index(1, 1, 1)));
+  const T rw = mul_(r, w), bw = mul_(b, w), rv = mul_(vr, w), bv = mul_(vb, w);
+  pair(tensor_index(1, 1, 1), rw, bw, rv, bv, add_(sxy, u2));
+  pair(tensor_index(1, 1, -1), rw, bw, rv, bv, sub_(sxy, u2));
+  pair(tensor_index(1, -1, 1), rw, bw, rv, bv, add_(dxy, u2));
+  pair(tensor_index(1, -1, -1), rw, bw, rv, bv, sub_(dxy, u2));
+}
+
 // f^k = f^{k(e)}(rho_k, u, alpha_k), Phi = 0; written in layout 0.
 template <class Store>
 __global__ void k_init(Store st, Geom G, const __grid_constant__ KConst<typename DensOf<Store>::real> K,
                        const double* __restrict__ rr, const double* __restrict__ rb, const double* __restrict__ u) {
   using R = typename DensOf<Store>::real;
+  using T = typename WideOf<R>::type;
   const int64_t N = (int64_t)G.nx * G.ny * G.nz;
   const int64_t n = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (n >= N) return;
   const int x = (int)(n % G.nx), y = (int)((n / G.nx) % G.ny), z = (int)(n / ((int64_t)G.nx * G.ny));
-  const double u0 = u ? u[n] : 0.0, u1 = u ? u[N + n] : 0.0, u2 = u ? u[2 * N + n] : 0.0;
-  const double uu = u0 * u0 + u1 * u1 + u2 * u2;
-  const double r = rr[n], b = rb[n];
-  const double ar = K.alpha_r_d, ab = 8.0 / 27.0;
   const int64_t sn = snode(G, x, y, z);
-#pragma unroll
-  for (int t = 0; t < 27; ++t) {  // the lattice constants fold at compile time
-    const double w = weight_of(t);
-    const double cu = cx_of(t) * u0 + cy_of(t) * u1 + cz_of(t) * u2;
-    const double poly = w * (3.0 * cu + 4.5 * cu * cu - 1.5 * uu);
-    const double vr = t == REST ? ar : 27.0 / 19.0 * (1.0 - ar) * w;
-    const double vb = t == REST ? ab : 27.0 / 19.0 * (1.0 - ab) * w;
-    store_pair(st, K, sn, t, (R)(r * (vr + poly)), (R)(b * (vb + poly)));
-  }
+  equilibrium_pairs<T>(rr[n], rb[n], u ? u[n] : 0.0, u ? u[N + n] : 0.0, u ? u[2 * N + n] : 0.0, K.alpha_r_d,
+                       [&](int t, T fr, T fb) { store_pair(st, K, sn, t, (R)narrow_(fr), (R)narrow_(fb)); });
 }
 
 // one direction (paper order pdir) of the canonical [2][27][N] FP64 array <-> storage
@@ -1883,6 +1921,18 @@ __global__ void k_top_from_state(Store st, Geom G, const __grid_constant__ KCons
   }
 }
 
+// u = (j + F/2) / rho (Eq. Momentum) of node n into the three components of u
+template <typename T, typename R>
+__device__ __forceinline__ void write_velocity(const KConst<R>& K, T rho, const T j[3], double* __restrict__ u,
+                                               int64_t n, int64_t N) {
+  T k = wide_<T>(0.0);
+  if (K.force_mode == FORCE_BUOYANCY || K.force_mode == FORCE_DISPERSED) k = sub_(rho, wide_<T>((double)K.rho_ref));
+  else if (K.force_mode == FORCE_UNIFORM) k = wide_<T>(1.0);
+#pragma unroll
+  for (int a = 0; a < 3; ++a)
+    u[a * N + n] = to_f64(div_(mad_(k, wide_<T>(0.5 * (double)K.g[a]), j[a]), rho));
+}
+
 // rho_r, rho_b, u (Eq. Momentum) into FP64 device buffers (any may be null)
 template <class Store>
 __global__ void k_macro(Store st, Geom G, const __grid_constant__ KConst<typename DensOf<Store>::real> K, int layout,
@@ -1902,26 +1952,33 @@ __global__ void k_macro(Store st, Geom G, const __grid_constant__ KConst<typenam
     slot_of(nm, layout, t, node, dir);
     st.load_rb(node, dir, speed2_of(t), K, fr[t], fb[t]);
   }
-  double r = 0.0, b = 0.0, j[3] = {0.0, 0.0, 0.0};
+  using T = typename WideOf<R>::type;
+  T sr = wide_<T>(0.0), sb = wide_<T>(0.0);
 #pragma unroll
   for (int t = 0; t < 27; ++t) {
-    r += (double)fr[t];
-    b += (double)fb[t];
-    const double s = (double)fr[t] + (double)fb[t];
-    j[0] += cx_of(t) * s;
-    j[1] += cy_of(t) * s;
-    j[2] += cz_of(t) * s;
+    acc_(sr, fr[t]);
+    acc_(sb, fb[t]);
   }
-  const double rho = r + b;
-  double k = 0.0;
-  if (K.force_mode == FORCE_BUOYANCY || K.force_mode == FORCE_DISPERSED) k = rho - (double)K.rho_ref;
-  else if (K.force_mode == FORCE_UNIFORM) k = 1.0;
-  if (rr) rr[n] = r;
-  if (rb) rb[n] = b;
+  if (rr) rr[n] = to_f64(sr);
+  if (rb) rb[n] = to_f64(sb);
   if (u) {
-    u[n] = (j[0] + 0.5 * k * (double)K.g[0]) / rho;
-    u[N + n] = (j[1] + 0.5 * k * (double)K.g[1]) / rho;
-    u[2 * N + n] = (j[2] + 0.5 * k * (double)K.g[2]) / rho;
+    // momentum from the 13 differences of opposite populations
+    T m[3] = {wide_<T>(0.0), wide_<T>(0.0), wide_<T>(0.0)};
+#pragma unroll
+    for (int t = 14; t < 27; ++t) {
+      T d = wide_<T>(0.0);
+      acc_(d, fr[t]);
+      acc_(d, -fr[26 - t]);
+      acc_(d, fb[t]);
+      acc_(d, -fb[26 - t]);
+      const int c[3] = {cx_of(t), cy_of(t), cz_of(t)};
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        if (c[a] > 0) acc_(m[a], d);
+        if (c[a] < 0) acc_(m[a], neg_(d));
+      }
+    }
+    write_velocity(K, add_(sr, sb), m, u, n, N);
   }
 }
 
@@ -1949,15 +2006,28 @@ static __global__ void __launch_bounds__(DIAG_THREADS) k_diag_partial(Geom G, do
   const int64_t N = (int64_t)G.nx * G.ny * G.nz;
   const int64_t plane = (int64_t)G.nx * G.ny;
   double acc[DIAG_VALS] = {0, 0, 0, 0, 0, 0, -1.0};
+  int n_in = 0, n_out = 0;
   const double cr = 9.0 * (1.0 - alpha_r) / 19.0, cb = 9.0 * (1.0 - alpha_b) / 19.0;
   for (int64_t n = blockIdx.x * (int64_t)DIAG_THREADS + threadIdx.x; n < N; n += (int64_t)gridDim.x * DIAG_THREADS) {
     const double r = rr[n], b = rb[n];
-    const double rho = r + b, phi = (r - b) / rho;
+    const double rho = r + b, d = r - b;
     acc[0] += r;
     acc[1] += b;
-    const double p = r * cr + b * cb;
-    if (phi > 0.99) { acc[2] += p; acc[3] += 1.0; }
-    if (phi < -0.99) { acc[4] += p; acc[5] += 1.0; }
+    // phi = d / rho against 0.99, -0.99 and 0.  FP64 issues at 1/64 of the FP32 rate, so the FP32
+    // quotient (within 2^-22 of phi) decides wherever it lies more than 1e-6 from a threshold, and
+    // only the other nodes, and those with phi > 0, divide in FP64: the same decisions
+    const float q = __fdiv_rn((float)d, (float)rho);
+    const bool sure = fabsf((float)rho) > 1e-30f && fabsf(q - 0.99f) > 1e-6f && fabsf(q + 0.99f) > 1e-6f &&
+                      fabsf(q) > 1e-6f;
+    const double phi = sure && q < 0.f ? (double)q : d / rho;
+    if (phi > 0.99) {
+      acc[2] += r * cr + b * cb;
+      ++n_in;
+    }
+    if (phi < -0.99) {
+      acc[4] += r * cr + b * cb;
+      ++n_out;
+    }
     if (phi > 0.0) {
       const int z = (int)(n / plane);
       double cand = (double)z;
@@ -1969,6 +2039,8 @@ static __global__ void __launch_bounds__(DIAG_THREADS) k_diag_partial(Geom G, do
       acc[6] = fmax(acc[6], cand);
     }
   }
+  acc[3] = n_in;
+  acc[5] = n_out;
   __shared__ double sh[DIAG_VALS][DIAG_THREADS / 32];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
 #pragma unroll

@@ -1,0 +1,59 @@
+"""Initial populations and macroscopic fields: FP32-arithmetic storages take FP64 fields in and out
+through head + tail FP32 pairs.
+
+Bounds.  A pair holds 48 bits and each operation on pairs errs by a few units of 2^-47 of its
+operands, so an initial FP32 population is the FP64 value (a sum of terms at most 8 times its size
+for |u| <= 0.15) rounded once: 2^-24 of it, plus 2^-40.  A macroscopic density, a sum of 27 stored
+values, errs by less than 27 * 2^-46 < 2^-41 of it; the velocity, from 54 values and one quotient,
+by less than 2^-40 of the largest possible speed 1.  FP64 storage: 2^-48 for all.
+"""
+import numpy as np
+import pytest
+
+import lbm_inputs as L
+import oracle
+import paper_1705_03141_gb300 as pkg
+
+pytestmark = pytest.mark.gpu
+
+# one node deep, odd, one row of a whole block plus one node, several blocks of threads
+SHAPES = [(3, 3, 3), (33, 5, 4), (32, 9, 7), (65, 8, 6)]
+C = None
+
+
+def _work(shape):
+    p = dict(L.parity_cases()[3][1]["params"])  # the jet's densities and force
+    p.update(bc=(0,) * 6, inflow=None)
+    return dict(name="box", shape=shape, params=p, fields=("random_blobs", dict(seed=3, blobs=2)), steps=0)
+
+
+@pytest.mark.parametrize("shape", SHAPES)
+@pytest.mark.parametrize("storage,eps_f,eps_m", [("f64", 2.0 ** -48, 2.0 ** -48), ("f32", 2.0 ** -24 + 2.0 ** -40, 2.0 ** -40),
+                                                 ("f16", None, 2.0 ** -40), ("bf16", None, 2.0 ** -40)])
+def test_initial_populations_and_macroscopic_sums(shape, storage, eps_f, eps_m):
+    w = _work(shape)
+    rr, rb, u = L.initial_fields(w, seed=5, u_amp=0.1)
+    lat = pkg.Lattice(shape, w["params"], storage=storage)
+    lat.init_fields(rr, rb, u)
+    f = lat.get_populations()
+    orc = oracle.Oracle(shape, w["params"])
+    orc.init_fields(rr, rb, u)
+    ref = orc.f.reshape(f.shape)
+    if eps_f is not None:
+        assert np.all(np.abs(f - ref) <= eps_f * np.abs(ref) + 1e-45)
+    r, b, v = lat.macro()
+    lat.close()
+    # the same sums of the stored populations in extended precision
+    g = f.astype(np.longdouble)
+    sr, sb = g[0].sum(0), g[1].sum(0)
+    assert np.all(np.abs(r - sr) <= eps_m * sr + 1e-45) and np.all(np.abs(b - sb) <= eps_m * sb + 1e-45)
+    c = oracle.tables()[0]
+    c = np.asarray(c).reshape(27, 3)
+    p = w["params"]
+    rho = sr + sb
+    # the force's constants are held in the storage's compute type
+    real = np.float64 if storage == "f64" else np.float32
+    for a in range(3):
+        mom = sum(int(c[i][a]) * (g[0, i] + g[1, i]) for i in range(27))
+        F = (rho - np.longdouble(real(p["rho_b0"]))) * np.longdouble(real(p["g"][a]))
+        assert np.all(np.abs(v[a] - (mom + F / 2) / rho) <= 4 * eps_m)
