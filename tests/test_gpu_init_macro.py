@@ -18,7 +18,6 @@ pytestmark = pytest.mark.gpu
 
 # one node deep, odd, one row of a whole block plus one node, several blocks of threads
 SHAPES = [(3, 3, 3), (33, 5, 4), (32, 9, 7), (65, 8, 6)]
-C = None
 
 
 def _work(shape):

@@ -1,0 +1,96 @@
+"""The fused network kernels at the edges of their shapes against the FP64 reference MLP.
+
+Fused: widths that are multiples of 64 up to 256, n_in <= 64, n_out <= 256; a batch tile has 16 rows (32 above
+2432 rows), a weight-gradient split 256.  The last two shapes run layer by layer.  The reference takes
+the same bfloat16-rounded weights and inputs, so what differs is the bfloat16 rounding (relative 2^-9)
+of each hidden activation and each backward signal: 1e-2 of max|y| on outputs, as derived in
+tests/test_gpu_mlp.py for four hidden layers.  A gradient is a sum over the batch of products
+d(b, o) h(b, i) whose factors each carry such relative errors, a few 2^-9 after several layers, so its error is
+bounded by 3e-2 = 15 * 2^-9 of the sum of the products' magnitudes (the sum itself cancels: with
+random labels its size falls like batch^-1/2 while the rounding of the factors is common to the rows).
+"""
+import numpy as np
+import pytest
+
+import paper_1705_03141_gb300 as pkg
+from oracle import mlp_oracle as M
+
+pytestmark = pytest.mark.gpu
+
+# n_in, width, depth, n_pos, n_cls, batch
+SHAPES = [(5, 256, 4, 64, 4, 1), (5, 256, 4, 64, 4, 17), (5, 256, 4, 64, 4, 64), (5, 256, 4, 64, 4, 2433),
+          (1, 64, 1, 1, 0, 16), (64, 128, 2, 0, 3, 33), (7, 192, 3, 63, 2, 257), (3, 256, 1, 252, 4, 31),
+          (5, 64, 8, 9, 4, 48), (5, 96, 2, 8, 4, 40), (65, 128, 2, 8, 4, 40)]
+
+
+def bf16(a):
+    u = np.asarray(a, dtype=np.float32).view(np.uint32).astype(np.uint64)
+    return (((u + 0x7FFF + ((u >> 16) & 1)) & 0xFFFF0000).astype(np.uint32)).view(np.float32).astype(np.float64)
+
+
+@pytest.mark.parametrize("n_in,width,depth,n_pos,n_cls,batch", SHAPES)
+def test_forward_gradient_and_step(cuda, n_in, width, depth, n_pos, n_cls, batch):
+    import torch
+
+    sizes = [n_in] + [width] * depth + [n_pos + n_cls]
+    flat = M.flatten(M.init_params(sizes, seed=3)).astype(np.float32)
+    net = pkg.Mlp(n_in=n_in, width=width, depth=depth, n_pos=n_pos, n_cls=n_cls, max_batch=batch)
+    net.set_params(flat)
+    ref = [(bf16(W), b.astype(np.float32).astype(np.float64)) for W, b in M.unflatten(flat.astype(np.float64), sizes)]
+    rng = np.random.default_rng(4)
+    x = rng.uniform(-1, 1, size=(batch, n_in)).astype(np.float32)
+    t = (0.3 * rng.normal(size=(batch, n_pos))).astype(np.float32)
+    lab = rng.integers(0, max(n_cls, 1), size=batch).astype(np.int32)
+    y = net.forward(x)
+    yr, cache = M.forward(ref, bf16(x))
+    assert np.max(np.abs(y - yr)) < 1e-2 * np.max(np.abs(yr))
+    xd = torch.from_numpy(x).cuda()
+    np.testing.assert_array_equal(net.forward(xd).cpu().numpy(), y)  # the caller's device buffers, no staging
+    # loss and gradient: positions and classes may be absent
+    dy = np.zeros_like(yr)
+    want = 0.0
+    if n_pos:
+        d = yr[:, :n_pos] - t
+        want += np.mean(d * d)
+        dy[:, :n_pos] = 2.0 * d / d.size
+    if n_cls:
+        z = yr[:, n_pos:] - yr[:, n_pos:].max(axis=1, keepdims=True)
+        p = np.exp(z) / np.exp(z).sum(axis=1, keepdims=True)
+        want += 0.5 * -np.mean(np.log(p[np.arange(batch), lab]))
+        dy[:, n_pos:] = 0.5 * (p - np.eye(n_cls)[lab]) / batch
+    gr = M.flatten(M.backward(ref, cache, dy))
+    mags, d = [], dy  # per layer the sums of |d| |h| behind its weight and bias gradients
+    for l in range(len(ref) - 1, -1, -1):
+        h, z = cache[l]
+        if l < len(ref) - 1:
+            d = d * M.silu_grad(z)
+        mags.insert(0, (np.abs(d).T @ np.abs(h), np.abs(d).sum(0)))
+        d = d @ ref[l][0]
+    mag = M.flatten(mags)
+    loss, g = net.loss_grad(x, t, lab, w_pos=1.0, w_cls=0.5)
+    assert loss == pytest.approx(want, rel=1e-2, abs=1e-6)
+    o = 0
+    for a, b in zip(sizes[:-1], sizes[1:]):
+        for n in (a * b, b):
+            assert np.max(np.abs(g[o:o + n] - gr[o:o + n])) < 3e-2 * np.max(mag[o:o + n]) + 1e-9, (a, b, n)
+            o += n
+    loss2, g2 = net.loss_grad(x, t, lab, w_pos=1.0, w_cls=0.5)
+    assert loss2 == loss
+    np.testing.assert_array_equal(g2, g)
+    # the first Adam step from this gradient moves every parameter by lr g / (|g| + 1e-8)
+    assert net.train_step(x, t, lab, lr=1e-2, w_pos=1.0, w_cls=0.5) == loss
+    step = net.get_params() - flat
+    np.testing.assert_allclose(step, -1e-2 * g / (np.abs(g) + 1e-8), rtol=0, atol=1e-2 * 2e-4 + 2.0 ** -23)
+    # the bfloat16 copies follow the parameters, the transposed one among them
+    fresh = pkg.Mlp(n_in=n_in, width=width, depth=depth, n_pos=n_pos, n_cls=n_cls, max_batch=batch)
+    fresh.set_params(net.get_params())
+    la, ga = net.loss_grad(x, t, lab)
+    lb, gb = fresh.loss_grad(x, t, lab)
+    assert la == lb
+    np.testing.assert_array_equal(ga, gb)
+    if n_cls:  # a label out of range is reported, and the next call is clean
+        with pytest.raises(pkg.LbmError):
+            net.loss_grad(x, t, np.full(batch, n_cls, np.int32))
+        assert net.loss_grad(x, t, lab)[0] == la
+    net.close()
+    fresh.close()
