@@ -68,7 +68,7 @@ def peaks():
 
 
 KERNEL_SOURCES = ("lbm_f2.cuh", "lbm_kernels.cuh", "lbm_kernels_f16.cu", "lbm_kernels_f32.cu", "lbm_kernels_f64.cu",
-                  "lbm_lattice.cuh", "lbm_launch.cuh", "lbm_compact.cuh", "lbm_kernels_c16.cu", "lbm_tma.cuh",
+                  "lbm_lattice.cuh", "lbm_launch.cuh", "lbm_compact.cuh", "lbm_df.cuh", "lbm_kernels_c16.cu", "lbm_tma.cuh",
                   "lbm_pipe.cuh")
 
 
