@@ -380,22 +380,25 @@ lbm_status lbm_create(int nx, int ny, int nz, const lbm_params* p, lbm** out) {
   int64_t Ns = 0;
   h->L = plan(nx, ny, nz, p, h->ks, &Ns, &h->diag_blocks);
   h->stream = static_cast<cudaStream_t>(p->cuda_stream);
-  // default, as measured on GB300: FP32 storage runs the fused density pass when rows
-  // fill whole 32-node blocks (its collide-stream kernel is bandwidth-bound, so dropping
-  // the separate density pass pays; partial blocks would take the per-direction atomic
-  // path); the packed storages run the two-pass scheme with the TMA-pipelined collide-stream
+  // default, as measured on GB300: FP32 storage runs the fused density pass (its collide-stream
+  // kernel is bandwidth-bound, so dropping the separate density pass pays) when rows fill whole
+  // 32-node blocks, and with ragged rows from a million nodes on, where the populations no longer
+  // fit in L2 (us a step, fused against two passes: 200x200x500 2048 / 2277, 100x90x300 361 / 378,
+  // 80x80x320 234 / 242, but 85^3 79.7 / 77.3, 41^3 19.2 / 15.5); the packed storages run the
+  // two-pass scheme with the TMA-pipelined collide-stream
   // kernel on the interior tiles (variant 5: 0.384 against 0.394 ms for the one-node kernel on
   // the 128x128x512 jet; it runs variant 1 where it does not apply) and FP64 one node per
-  // thread (the packed kernels are issue-bound, and the fused accumulation costs more
-  // instructions than the density pass); the two-node kernel's register footprint
-  // leaves 8 warps per SM and measured slower everywhere
+  // thread (the fused accumulation costs the packed kernels more than the density pass); the two-node
+  // kernel's register footprint leaves 8 warps per SM and measured slower everywhere
   h->halo = p->bc[4] == LBM_BC_HALO || p->bc[5] == LBM_BC_HALO;
   h->half = 0;
   h->recs_valid = false;
   h->dens_ready = false;
   const bool packed = p->storage == LBM_STORE_F16 || p->storage == LBM_STORE_BF16;
   h->variant = p->variant != 0 ? p->variant
-                               : (p->storage == LBM_STORE_F32 && nx % 32 == 0 && !h->halo ? 3 : (packed ? 5 : 1));
+                               : (p->storage == LBM_STORE_F32 && (nx % 32 == 0 || h->N >= (1 << 20)) && !h->halo
+                                      ? 3
+                                      : (packed ? 5 : 1));
   h->fix_ready = false;
   // block shape: as measured on GB300 (128x128x512 jet), the fused FP32 kernel runs fastest in
   // 32x2x4 blocks (0.784 against 0.814 ms for 32x4x2); every other kernel in 32x4x2

@@ -26,6 +26,7 @@
 #include <cuda_runtime.h>
 #include <cuda_fp16.h>
 #include <cuda_bf16.h>
+#include <math.h>
 #include <stdint.h>
 
 #include <type_traits>
@@ -97,6 +98,7 @@ struct KConst {
   // packed storage: rest-state value of a direction of speed class s (|c|^2 = s)
   // at red fraction q is refB[s] + q * dref[s]; dref is zero for moving classes.
   R refB[4], dref[4];
+  R fix_scale, fix_inv;    // fused density pass: 2^e and 2^-e (make_kconst)
   // inlet (noise in FP64 so that both precisions draw the same variates)
   double rho_r0_d, alpha_r_d, u_j0, noise_frac;
   uint64_t seed;
@@ -126,6 +128,13 @@ inline KConst<R> make_kconst(const Phys& P) {
     K.refB[s] = (R)rb;
     K.dref[s] = (R)(s == 0 ? rr - rb : 0.0);  // equal for moving classes (gamma = (1-alpha_b)/(1-alpha_r))
   }
+  // fixed-point densities: 2^-25 of the power of two at or above the larger phase density (the
+  // rounding of an FP32 density of that size), never coarser than 2^-22
+  int e = 25 - (int)ceil(log2(P.rho_r0 > P.rho_b0 ? P.rho_r0 : P.rho_b0));
+  if (e < 22) e = 22;
+  if (e > 28) e = 28;
+  K.fix_scale = (R)ldexp(1.0, e);
+  K.fix_inv = (R)ldexp(1.0, -e);
   K.rho_r0_d = P.rho_r0;
   K.alpha_r_d = P.alpha_r;
   K.u_j0 = P.u_j0;
@@ -615,7 +624,8 @@ struct Recol {
 // (Eq. scoll with Eqs. ketF-ketFd), M = T V3 (V3: raw moments, T: the sparse map
 // of Eq. momentSet): one forward cascade, the relaxation of each parity class of raw moments with
 // the closed-form moments of f^(e) - F'/2 and F' + Omega^(2) (relax_moments), one inverse cascade.
-template <typename R>
+// FOLD: the form of relax_moments.
+template <bool FOLD, typename R>
 __device__ __forceinline__ Recol<R> collide(const KConst<R>& K, const R rho_r, const R ft[27], const R gphi[3],
                                             const R grho[3], R f[27]) {
 #pragma unroll
@@ -650,7 +660,7 @@ __device__ __forceinline__ Recol<R> collide(const KConst<R>& K, const R rho_r, c
   out.n2 = G2 * inv_gn;
   const R m_abs = K.A29 * gg * inv_gn;  // (2/9) A |grad phi|
   const R n[3] = {out.n0, out.n1, out.n2}, m[3] = {m_abs * out.n0, m_abs * out.n1, m_abs * out.n2};
-  relax_moments(K.rx, f, s_sh, Beq, u, w, F, m_abs, m, n);
+  relax_moments<FOLD>(K.rx, f, s_sh, Beq, u, w, F, m_abs, m, n);
   raw_inverse(f);  // f holds f*
 
   const R abar = K.a_mid + K.a_half * phi;
@@ -703,18 +713,17 @@ __device__ __forceinline__ int tile_zmax(const Geom& G) { return G.bc[5] == BC_H
 // (boundaries: y is the owner of the slot S(x, i)), so the collide-stream
 // kernel of step t can accumulate the next step's (rho, rho_r) while it writes
 // f*, and the separate density pass (which rereads every population) is not
-// needed.  Accumulators are fixed point, value * 2^22 (resolution 2.4e-7):
-// integer addition is exact and associative, so the atomics of different
-// blocks give bitwise reproducible sums in any order.  One 64-bit word per node
-// holds both, rho_r * 2^54 + rho * 2^22 in two's complement: every partial sum
-// is added as one 64-bit integer, and since the total rho * 2^22 lies in
-// [0, 2^32) (rho < 1024), the low 32 bits return rho and the high 32 bits
-// rho_r (|rho_r| < 512) exactly, whatever the signs of the partial sums.
-constexpr float kFixScale = 4194304.0f;
-constexpr float kFixInv = 1.0f / 4194304.0f;
-__device__ __forceinline__ int to_fix(float v) { return __float2int_rn(v * kFixScale); }
-__device__ __forceinline__ unsigned long long pack_fix(float rho, float rho_r) {
-  return ((unsigned long long)(unsigned)to_fix(rho_r) << 32) + (unsigned long long)(long long)to_fix(rho);
+// needed.  Accumulators are fixed point, value * 2^e with e = 25 for densities up to 1, 22 for
+// densities up to 64 (KConst::fix_scale): integer addition is exact and associative, so the atomics
+// of different blocks give bitwise reproducible sums in any order.  One 64-bit word per node
+// holds both, rho_r * 2^(e + 32) + rho * 2^e in two's complement: every partial sum
+// is added as one 64-bit integer, and since the total rho * 2^e lies in
+// [0, 2^32) (rho < 64 times the reference density, at least 8 times 64), the low 32 bits return rho and the
+// high 32 bits rho_r exactly, whatever the signs of the partial sums.
+__device__ __forceinline__ int to_fix(float v, float scale) { return __float2int_rn(v * scale); }
+__device__ __forceinline__ unsigned long long pack_fix(float rho, float rho_r, float scale) {
+  return ((unsigned long long)(unsigned)to_fix(rho_r, scale) << 32) +
+         (unsigned long long)(long long)to_fix(rho, scale);
 }
 
 struct FusedIO {
@@ -725,9 +734,9 @@ struct FusedIO {
 
 // (rho, phi) of a density-tile cell from the fixed-point accumulators; the
 // Dirichlet inlet nodes carry rho_r0 and phi = 1 (as in pass 1)
-__device__ __forceinline__ float2 fused_cell(const FusedIO& io, int64_t i) {
+__device__ __forceinline__ float2 fused_cell(const FusedIO& io, int64_t i, float inv) {
   const unsigned long long v = io.cur[i];
-  const float rho = (float)(unsigned)v * kFixInv, rr = (float)(int)(unsigned)(v >> 32) * kFixInv;
+  const float rho = (float)(unsigned)v * inv, rr = (float)(int)(unsigned)(v >> 32) * inv;
   return make_float2(rho, __fdividef(rr + rr - rho, rho));
 }
 
@@ -745,32 +754,33 @@ __device__ __forceinline__ R red_part(R fstar, const Recol<R>& rc) {
   return fma_(rc.rc[speed2_of(T)], cdot<T>(rc.n0, rc.n1, rc.n2), rc.frac * fstar);
 }
 
-// Fast rows (a warp is one x-row whose y/z neighbours are inside the box, all
-// lanes active): the directions (-1|0|+1, dy, dz) = 3K, 3K+1, 3K+2 of the warp
+// Fast rows (a warp is one x-row whose y/z neighbours are inside the box; its lanes
+// 0 .. last hold nodes): the directions (-1|0|+1, dy, dz) = 3K, 3K+1, 3K+2 of the warp
 // all land in the target row (y+dy, z+dz); lane l's target x0+l collects
-// z(l) + p(l-1) + m(l+1), summed with two shuffles; lanes 0 and 31 also write
-// m(0) / p(31) into the edge columns.
+// z(l) + p(l-1) + m(l+1), summed with two shuffles; lanes 0 and `last` also write
+// m(0) / p(last) into the columns beside the row.
 template <int K, bool RECOL, typename R, int BYv = BY, int TXv = TX>
-__device__ __forceinline__ void fused_row(float2* prow, const R f[27], const Recol<R>& rc) {
+__device__ __forceinline__ void fused_row(float2* prow, int last, const R f[27], const Recol<R>& rc) {
   const int lane = threadIdx.x;
+  const unsigned mask = 0xffffffffu >> (31 - last);
   const float mt = f[3 * K], zt = f[3 * K + 1], pt = f[3 * K + 2];
   const float mr = red_part<3 * K, RECOL>(f[3 * K], rc), zr = red_part<3 * K + 1, RECOL>(f[3 * K + 1], rc),
               pr = red_part<3 * K + 2, RECOL>(f[3 * K + 2], rc);
-  const float pt_in = __shfl_up_sync(0xffffffffu, pt, 1), pr_in = __shfl_up_sync(0xffffffffu, pr, 1);
-  const float mt_in = __shfl_down_sync(0xffffffffu, mt, 1), mr_in = __shfl_down_sync(0xffffffffu, mr, 1);
+  const float pt_in = __shfl_up_sync(mask, pt, 1), pr_in = __shfl_up_sync(mask, pr, 1);
+  const float mt_in = __shfl_down_sync(mask, mt, 1), mr_in = __shfl_down_sync(mask, mr, 1);
   float st = zt, sr = zr;
   if (lane > 0) {
     st += pt_in;
     sr += pr_in;
   }
-  if (lane < 31) {
+  if (lane < last) {
     st += mt_in;
     sr += mr_in;
   }
   float2* row = prow + (((threadIdx.y + BYv * threadIdx.z) * 9 + K) * TXv);
   row[lane + 1] = make_float2(st, sr);
   if (lane == 0) row[0] = make_float2(mt, mr);
-  if (lane == 31) row[TXv - 1] = make_float2(pt, pr);
+  if (lane == last) row[last + 2] = make_float2(pt, pr);
 }
 
 // target coordinate along one axis of the slot S(x, t) (c: the component of c_t)
@@ -794,8 +804,8 @@ __device__ __forceinline__ void axis_target(int& q, int p, int c, int n, int bc_
 // (bounced back to x, reflected, wrapped, or into the ghost plane above an
 // outflow face, which no node reads as a density).
 template <int T, typename R>
-__device__ __forceinline__ void fused_node(const Geom& G, const FusedIO& io, int x, int y, int z, const R f[27],
-                                           const Recol<R>& rc) {
+__device__ __forceinline__ void fused_node(const Geom& G, const FusedIO& io, R scale, int x, int y, int z,
+                                           const R f[27], const Recol<R>& rc) {
   constexpr int dx = cx_of(T), dy = cy_of(T), dz = cz_of(T);
   int tx = x + dx, ty = y + dy, tz = z + dz;
   bool bounce = false, ghost = false;
@@ -809,7 +819,7 @@ __device__ __forceinline__ void fused_node(const Geom& G, const FusedIO& io, int
   } else if (ghost) {
     return;
   }
-  atomicAdd(io.nxt + dnode(G, tx, ty, tz), pack_fix((float)f[T], (float)red_part<T, true>(f[T], rc)));
+  atomicAdd(io.nxt + dnode(G, tx, ty, tz), pack_fix((float)f[T], (float)red_part<T, true>(f[T], rc), scale));
 }
 
 // grad phi and grad rho at tile cell (lx, ly, lz) from the (rho, phi) halo tile:
@@ -929,9 +939,9 @@ struct EmitLoop {
     emit<T, FAST, RECOL, ODDT>(st, K, G, nm, ar, odd, f, rc);
     if constexpr (FUSED) {
       if constexpr (FAST) {
-        if constexpr (T % 3 == 2) fused_row<T / 3, RECOL, R, BYv, TXv>(prow, f, rc);
+        if constexpr (T % 3 == 2) fused_row<T / 3, RECOL, R, BYv, TXv>(prow, min(31, G.nx - 1 - (x - (int)threadIdx.x)), f, rc);
       } else {
-        fused_node<T>(G, io, x, y, z, f, rc);
+        fused_node<T>(G, io, (R)K.fix_scale, x, y, z, f, rc);
       }
     }
     EmitLoop<T + 1, Store, R, FAST, RECOL, FUSED, ODDT, BYv, TXv>::run(st, K, G, nm, ar, odd, f, rc, prow, io, x, y, z);
@@ -1043,7 +1053,7 @@ __global__ void __launch_bounds__(B::NT, 4) k_density(Store st, Geom G,
   for (int t = 0; t < 27; ++t) rt += ft[t];
   if (!(rt > D(0)) || !(rt < D(1e30))) atomicOr(flag, 1);
   if constexpr (FIX) {
-    fix[dnode(G, x, y, z)] = pack_fix((float)rt, (float)rr);
+    fix[dnode(G, x, y, z)] = pack_fix((float)rt, (float)rr, (float)K.fix_scale);
   } else {
     D rb = rt - rr;
     if (is_inlet(G, x, y, z)) {
@@ -1238,9 +1248,8 @@ __global__ void __launch_bounds__(B::NT, MINB)
   }
 
   R rho_r = R(0), ft[27];
-  // a warp is one x-row of the block: the fast-row test is warp-uniform (the fused pass sums
-  // across the 32 lanes of a fast row, so there the row must also be complete in x)
-  const bool fast = fast_row(G, y, z) && (!FUSED || x0 + B::BX <= G.nx);
+  // a warp is one x-row of the block: the fast-row test is warp-uniform
+  const bool fast = fast_row(G, y, z);
   if (FUSED && threadIdx.x == 0) pfast[tid >> 5] = active && fast;
   if (active) {
     if (fast) {
@@ -1287,8 +1296,8 @@ __global__ void __launch_bounds__(B::NT, MINB)
         const int cy = gy < G.ny ? gy : G.ny - 1, cz = gz <= tile_zmax(G) ? gz : tile_zmax(G);
         const int64_t rbase = (int64_t)G.nx * ((int64_t)cy + (int64_t)G.ny * cz);
         if constexpr (FUSED) {
-          tile[row * B::TXT + 1 + lane] = fused_cell(io, rbase + cxa);
-          if (lane < B::TX - 32) tile[row * B::TXT + 33 + lane] = fused_cell(io, rbase + cxb);
+          tile[row * B::TXT + 1 + lane] = fused_cell(io, rbase + cxa, K.fix_inv);
+          if (lane < B::TX - 32) tile[row * B::TXT + 33 + lane] = fused_cell(io, rbase + cxb, K.fix_inv);
         } else {
           tile[row * B::TXT + 1 + lane] = dens[rbase + cxa];
           if (lane < B::TX - 32) tile[row * B::TXT + 33 + lane] = dens[rbase + cxb];
@@ -1332,7 +1341,7 @@ __global__ void __launch_bounds__(B::NT, MINB)
       rc.rho = R(1);
       rc.has_n = false;
     } else {
-      rc = collide(K, rho_r, ft, gphi, grho, f);
+      rc = collide<!std::is_same<Store, PlainStore<float>>::value>(K, rho_r, ft, gphi, grho, f);
     }
     if constexpr (FUSED) {
       // the watchdog of pass 1, on the density this step starts from
@@ -1370,10 +1379,13 @@ __global__ void __launch_bounds__(B::NT, MINB)
     // within one row of it; warp w takes tile rows w, w+8, w+16, lanes the columns
     __syncthreads();
     const int warp = tid >> 5, lane = threadIdx.x;
-    int gxa = x0 - 1 + lane, gxb = x0 + 31 + lane;  // lanes 0..1 also take columns 32, 33
+    // lanes 0..1 also take columns 32, 33; the columns beside the box belong to the node across a
+    // periodic face or, reflected, to the face node itself; columns further out hold nothing
+    int gxa = x0 - 1 + lane, gxb = x0 + 31 + lane;
+    const bool ina = gxa <= G.nx, inb = lane < B::TX - 32 && gxb <= G.nx;
     if (gxa < 0) gxa = G.bc[0] == BC_PERIODIC ? G.nx - 1 : 0;
-    if (gxb >= G.nx) gxb = G.bc[1] == BC_PERIODIC ? gxb - G.nx : G.nx - 1;
-    const bool ina = gxa < G.nx, inb = lane < B::TX - 32 && gxb >= 0 && gxb < G.nx;
+    if (gxa >= G.nx) gxa = G.bc[1] == BC_PERIODIC ? 0 : G.nx - 1;
+    if (gxb >= G.nx) gxb = G.bc[1] == BC_PERIODIC ? 0 : G.nx - 1;
 #pragma unroll
     for (int k = 0; k < (B::TY * B::TZ + B::NW - 1) / B::NW; ++k) {
       const int row = warp + k * B::NW;
@@ -1389,10 +1401,12 @@ __global__ void __launch_bounds__(B::NT, MINB)
               const int ky = ty - wy, kz = tz - wz;
               if (ky >= 0 && ky <= 2 && kz >= 0 && kz <= 2 && pfast[wy + B::BY * wz]) {
                 const float2* src = prow + ((wy + B::BY * wz) * 9 + ky + 3 * kz) * B::TX;
-                const float2 u = src[lane];
-                a.x += u.x;
-                a.y += u.y;
-                if (lane < B::TX - 32) {
+                if (ina) {
+                  const float2 u = src[lane];
+                  a.x += u.x;
+                  a.y += u.y;
+                }
+                if (inb) {
                   const float2 v = src[32 + lane];
                   b.x += v.x;
                   b.y += v.y;
@@ -1401,7 +1415,7 @@ __global__ void __launch_bounds__(B::NT, MINB)
             }
           }
           const int64_t rb = (int64_t)G.nx * ((int64_t)gy + (int64_t)G.ny * gz);
-          const unsigned long long av = pack_fix(a.x, a.y), bv = pack_fix(b.x, b.y);
+          const unsigned long long av = pack_fix(a.x, a.y, K.fix_scale), bv = pack_fix(b.x, b.y, K.fix_scale);
           if (ina && av) atomicAdd(io.nxt + rb + gxa, av);
           if (inb && bv) atomicAdd(io.nxt + rb + gxb, bv);
         }
@@ -1542,7 +1556,7 @@ __global__ void __launch_bounds__(NTHREADS, MINB)
         rc.rho = 1.0f;
         rc.has_n = false;
       } else {
-        rc = collide(K, rho_r, ft, gphi, grho, f);
+        rc = collide<true>(K, rho_r, ft, gphi, grho, f);
       }
       const bool recol = __any_sync(__activemask(), rc.has_n);
       const bool fast = fast_row(G, y, z);
@@ -1697,7 +1711,7 @@ __global__ void __launch_bounds__(PTHREADS, MINB)
   }
 
   F2 f[27];
-  Recol<F2> rc = collide(K, rho_r, ft, gphi, grho, f);
+  Recol<F2> rc = collide<false>(K, rho_r, ft, gphi, grho, f);
   if (z == 0 && G.inflow) {
     // Dirichlet inlet nodes (Sec. IV.A) replace the collision result lane by lane
 #pragma unroll
@@ -1794,7 +1808,7 @@ __global__ void __launch_bounds__(256) k_outflow(Store st, Geom G,
   // fused density pass: the plane's new populations replace what the collide-stream kernel accumulated
   if (fix) {
     const R sr = warp_allsum(nr), sa = warp_allsum(nr + nb);
-    if (lane == 0) fix[dnode(G, x, y, G.nz - 1)] = pack_fix((float)sa, (float)sr);
+    if (lane == 0) fix[dnode(G, x, y, G.nz - 1)] = pack_fix((float)sa, (float)sr, (float)K.fix_scale);
   }
 }
 

@@ -276,13 +276,16 @@ __host__ __device__ __forceinline__ void moment_forward(const R r[27], R m[27]) 
 template <typename R>
 struct RelaxConst {
   R s5h;               // s5 / 6
-  R q1, q2, q4, q2s;   // <b^2 c^2>: (1 - s19)/4, s19/12, (s19 - s17)/12, (s17 - s5)/9
+  R q1, q4, q2s;       // <b^2 c^2>: -s19/4, (s19 - s17)/12, (s17 - s5)/9
   R s19_6;             // s19 / 6
-  R t1, t2, t4, tb;    // <222>: (1 - s18)/8, S2 and S4 coefficients / 8, s18/72
-  R v1, v2, vj;        // <a b^2>: (1 - (s11 + s24)/2)/4, -(s11 - s24)/8, s11/12
-  R z1, z2, zj;        // <a b^2 c^2>: (1 - s14)/8, (s14 - s11)/12, j coefficient / 8
-  R p1, pt, pk;        // <a b c^2>: (1 - s21)/8, s21/48, s21/12
+  R t1, t2, t4;        // <222>: -s18/8, S2 and S4 coefficients / 8
+  R v1, v2;            // <a b^2>: -(s11 + s24)/8, -(s11 - s24)/8
+  R z1, z2;            // <a b^2 c^2>: -s14/8, (s14 - s11)/12
+  R p1, pk;            // <a b c^2>: -s21/8, s21/12
   R d1;                // <111>: (1 - s27)/8
+  // the folded form: (1 - s19)/4, s19/12, (1 - s18)/8, s18/72, (1 - (s11 + s24)/2)/4, s11/12,
+  // (1 - s14)/8, coefficient of j / 8, (1 - s21)/8, s21/48
+  R q1f, q2f, t1f, tbf, v1f, vjf, z1f, zjf, p1f, ptf;
 };
 
 // rate[j]: relaxation rate of moment j + 1 (the shear slots are not read)
@@ -292,25 +295,30 @@ inline RelaxConst<R> make_relax(const double rate[27]) {
                s21 = rate[20], s24 = rate[23], s27 = rate[26];
   RelaxConst<R> K;
   K.s5h = (R)(s5 / 6.0);
-  K.q1 = (R)((1.0 - s19) / 4.0);
-  K.q2 = (R)(s19 / 12.0);
+  K.q1 = (R)(-s19 / 4.0);
   K.q4 = (R)((s19 - s17) / 12.0);
   K.q2s = (R)((s17 - s5) / 9.0);
   K.s19_6 = (R)(s19 / 6.0);
-  K.t1 = (R)((1.0 - s18) / 8.0);
+  K.t1 = (R)(-s18 / 8.0);
   K.t2 = (R)(((s17 - s5) * 8.0 / 9.0 - (s18 - s5) * 4.0 / 9.0) / 8.0);
   K.t4 = (R)((s18 - s17) / 12.0);
-  K.tb = (R)(s18 / 72.0);
-  K.v1 = (R)((1.0 - 0.5 * (s11 + s24)) / 4.0);
+  K.v1 = (R)(-(s11 + s24) / 8.0);
   K.v2 = (R)(-(s11 - s24) / 8.0);
-  K.vj = (R)(s11 / 12.0);
-  K.z1 = (R)((1.0 - s14) / 8.0);
+  K.z1 = (R)(-s14 / 8.0);
   K.z2 = (R)((s14 - s11) / 12.0);
-  K.zj = (R)((s14 / 9.0 - (s14 - s11) * 4.0 / 9.0) / 8.0);
-  K.p1 = (R)((1.0 - s21) / 8.0);
-  K.pt = (R)(s21 / 48.0);
+  K.p1 = (R)(-s21 / 8.0);
   K.pk = (R)(s21 / 12.0);
   K.d1 = (R)((1.0 - s27) / 8.0);
+  K.q1f = (R)((1.0 - s19) / 4.0);
+  K.q2f = (R)(s19 / 12.0);
+  K.t1f = (R)((1.0 - s18) / 8.0);
+  K.tbf = (R)(s18 / 72.0);
+  K.v1f = (R)((1.0 - 0.5 * (s11 + s24)) / 4.0);
+  K.vjf = (R)(s11 / 12.0);
+  K.z1f = (R)((1.0 - s14) / 8.0);
+  K.zjf = (R)((s14 / 9.0 - (s14 - s11) * 4.0 / 9.0) / 8.0);
+  K.p1f = (R)((1.0 - s21) / 8.0);
+  K.ptf = (R)(s21 / 48.0);
   return K;
 }
 
@@ -326,12 +334,16 @@ inline RelaxConst<R> make_relax(const double rate[27]) {
 // pi_a = 2 u_a F_a + m_a n_a, m = (2/9) A |grad phi| n
 //   <a> = F_a,  <a^2> = pi_a - |m|,  <b^2c^2> = (sum pi - |m| - pi_a)/3,  <222> = (sum pi - |m|)/9,
 //   <ab> = u_a F_b + u_b F_a + m_a n_b = 3 <abc^2>,  <ab^2> = <ac^2> = 3 <ab^2c^2> = F_a/3.
-// About 170 operations; relaxing the 23 moments of Eq. (momentSet) one by one between T and T^-1,
-// with the closed forms added per raw moment, took about 330.  Measured with the gradients by
+// FOLD: each moment as a scaled moment plus a scaled equilibrium (about 170 operations); otherwise as
+// itself plus its change (about 190), which rounds it once at its own size.  FP32 storage takes the
+// second: folded, its fields came out 3 to 13 % further from FP64, against 15 % nearer than with
+// the moment-by-moment form below.  The 16-bit storages, whose own rounding is 2^12 times larger, and FP64
+// (7.5e-14 either way) take the first: 3 % of a step.
+// Relaxing the 23 moments of Eq. (momentSet) one by one between T and T^-1, with the closed forms
+// added per raw moment, took about 330 operations.  Measured with the gradients by
 // opposite pairs: collide-stream pass in FP64 on a 32^3 box (bound by the FP64 pipe) 69 -> 56 us;
-// packed half, interior tiles of a 128^3 jet (bound by instruction issue) 78 -> 72 us on even and
-// 88 -> 85 us on odd steps, 1048 -> 912 and 1210 -> 1089 instructions a node.
-template <typename R>
+// packed half, interior tiles of a 128^3 jet 78 -> 72 us on even and 88 -> 85 us on odd steps.
+template <bool FOLD, typename R>
 __host__ __device__ __forceinline__ void relax_moments(const RelaxConst<R>& K, R r[27], R s_sh, R B, const R u[3],
                                                        const R w[3], const R F[3], R m_abs, const R m[3],
                                                        const R n[3]) {
@@ -345,46 +357,99 @@ __host__ __device__ __forceinline__ void relax_moments(const RelaxConst<R>& K, R
   const R h0 = LBMK_R(2, 0, 0) - B - sg0, h1 = LBMK_R(0, 2, 0) - B - sg1, h2 = LBMK_R(0, 0, 2) - B - sg2;
   const R S2 = h0 + h1 + h2;
   const R S4 = LBMK_R(2, 2, 0) + LBMK_R(0, 2, 2) + LBMK_R(2, 0, 2) - fma_(R(2.0 / 3.0), tr, B);
-  const R c = fma_(R(-0.5), s_sh, R(0.5));                              // (1 - s)/2
-  const R L = fma_(fma_(R(1.0 / 6.0), s_sh, -K.s5h), S2, R(0.5) * (B - m_abs));
-  LBMK_R(2, 0, 0) = fma_(c, h0, fma_(R(0.5), sg0 + pi0, L));
-  LBMK_R(0, 2, 0) = fma_(c, h1, fma_(R(0.5), sg1 + pi1, L));
-  LBMK_R(0, 0, 2) = fma_(c, h2, fma_(R(0.5), sg2 + pi2, L));
   const R b = fma_(R(1.0 / 6.0), s_sh, -K.s19_6);                        // (s - s19)/6
   const R a2 = fma_(R(-1.0 / 3.0), b, K.q2s);
-  const R CQ = fma_(a2, S2, fma_(K.q4, S4, fma_(R(1.0 / 12.0), Z, K.q2 * Btr)));
-  LBMK_R(0, 2, 2) = fma_(K.q1, LBMK_R(0, 2, 2), fma_(b, h0, fma_(-K.q2, sg0, fma_(R(-1.0 / 12.0), pi0, CQ))));
-  LBMK_R(2, 0, 2) = fma_(K.q1, LBMK_R(2, 0, 2), fma_(b, h1, fma_(-K.q2, sg1, fma_(R(-1.0 / 12.0), pi1, CQ))));
-  LBMK_R(2, 2, 0) = fma_(K.q1, LBMK_R(2, 2, 0), fma_(b, h2, fma_(-K.q2, sg2, fma_(R(-1.0 / 12.0), pi2, CQ))));
-  LBMK_R(2, 2, 2) =
-      fma_(K.t1, LBMK_R(2, 2, 2), fma_(K.t4, S4, fma_(K.t2, S2, fma_(K.tb, Btr, R(1.0 / 72.0) * Z))));
-  // pairs <ab>, <abc^2>
-  const R c4 = R(0.5) * c, k = fma_(R(-1.0 / 12.0), s_sh, K.pk);         // (1 - s)/4, (s21 - s)/12
+  if constexpr (FOLD) {
+    const R c = fma_(R(-0.5), s_sh, R(0.5));                              // (1 - s)/2
+    const R L = fma_(fma_(R(1.0 / 6.0), s_sh, -K.s5h), S2, R(0.5) * (B - m_abs));
+    LBMK_R(2, 0, 0) = fma_(c, h0, fma_(R(0.5), sg0 + pi0, L));
+    LBMK_R(0, 2, 0) = fma_(c, h1, fma_(R(0.5), sg1 + pi1, L));
+    LBMK_R(0, 0, 2) = fma_(c, h2, fma_(R(0.5), sg2 + pi2, L));
+    const R CQ = fma_(a2, S2, fma_(K.q4, S4, fma_(R(1.0 / 12.0), Z, K.q2f * Btr)));
+    LBMK_R(0, 2, 2) = fma_(K.q1f, LBMK_R(0, 2, 2), fma_(b, h0, fma_(-K.q2f, sg0, fma_(R(-1.0 / 12.0), pi0, CQ))));
+    LBMK_R(2, 0, 2) = fma_(K.q1f, LBMK_R(2, 0, 2), fma_(b, h1, fma_(-K.q2f, sg1, fma_(R(-1.0 / 12.0), pi1, CQ))));
+    LBMK_R(2, 2, 0) = fma_(K.q1f, LBMK_R(2, 2, 0), fma_(b, h2, fma_(-K.q2f, sg2, fma_(R(-1.0 / 12.0), pi2, CQ))));
+    LBMK_R(2, 2, 2) =
+        fma_(K.t1f, LBMK_R(2, 2, 2), fma_(K.t4, S4, fma_(K.t2, S2, fma_(K.tbf, Btr, R(1.0 / 72.0) * Z))));
+    // pairs <ab>, <abc^2>
+    const R c4 = R(0.5) * c, k = fma_(R(-1.0 / 12.0), s_sh, K.pk);         // (1 - s)/4, (s21 - s)/12
 #define LBMK_PAIR(P, Q, x, y)                                                                       \
-  {                                                                                                 \
-    const R t = fma_(u[x], w[y], u[y] * w[x]);                                                      \
-    const R g = fma_(m[x], n[y], fma_(u[x], F[y], u[y] * F[x]));                                    \
-    const R h = fma_(R(-0.5), t, P);                                                                \
-    P = fma_(c4, h, fma_(R(0.125), t, R(0.25) * g));                                                \
-    Q = fma_(K.p1, Q, fma_(K.pt, t, fma_(k, h, R(1.0 / 24.0) * g)));                                \
-  }
-  LBMK_PAIR(LBMK_R(1, 1, 0), LBMK_R(1, 1, 2), 0, 1)
-  LBMK_PAIR(LBMK_R(0, 1, 1), LBMK_R(2, 1, 1), 1, 2)
-  LBMK_PAIR(LBMK_R(1, 0, 1), LBMK_R(1, 2, 1), 0, 2)
+    {                                                                                               \
+      const R t = fma_(u[x], w[y], u[y] * w[x]);                                                    \
+      const R g = fma_(m[x], n[y], fma_(u[x], F[y], u[y] * F[x]));                                  \
+      const R h = fma_(R(-0.5), t, P);                                                              \
+      P = fma_(c4, h, fma_(R(0.125), t, R(0.25) * g));                                              \
+      Q = fma_(K.p1f, Q, fma_(K.ptf, t, fma_(k, h, R(1.0 / 24.0) * g)));                            \
+    }
+    LBMK_PAIR(LBMK_R(1, 1, 0), LBMK_R(1, 1, 2), 0, 1)
+    LBMK_PAIR(LBMK_R(0, 1, 1), LBMK_R(2, 1, 1), 1, 2)
+    LBMK_PAIR(LBMK_R(1, 0, 1), LBMK_R(1, 2, 1), 0, 2)
 #undef LBMK_PAIR
-  // vectors <a>, <ab^2>, <ac^2>, <ab^2c^2>
+    // vectors <a>, <ab^2>, <ac^2>, <ab^2c^2>
 #define LBMK_VEC(J, P, Q, T, x)                                                                     \
-  {                                                                                                 \
-    const R j = J, e = fma_(K.vj, j, R(1.0 / 12.0) * F[x]), p = P, q = Q;                            \
-    J = R(0.5) * (j + F[x]);                                                                        \
-    P = fma_(K.v1, p, fma_(K.v2, q, e));                                                            \
-    Q = fma_(K.v1, q, fma_(K.v2, p, e));                                                            \
-    T = fma_(K.z1, T, fma_(K.z2, p + q, fma_(K.zj, j, R(1.0 / 72.0) * F[x])));                       \
-  }
-  LBMK_VEC(LBMK_R(1, 0, 0), LBMK_R(1, 2, 0), LBMK_R(1, 0, 2), LBMK_R(1, 2, 2), 0)
-  LBMK_VEC(LBMK_R(0, 1, 0), LBMK_R(0, 1, 2), LBMK_R(2, 1, 0), LBMK_R(2, 1, 2), 1)
-  LBMK_VEC(LBMK_R(0, 0, 1), LBMK_R(2, 0, 1), LBMK_R(0, 2, 1), LBMK_R(2, 2, 1), 2)
+    {                                                                                               \
+      const R j = J, e = fma_(K.vjf, j, R(1.0 / 12.0) * F[x]), p = P, q = Q;                         \
+      J = R(0.5) * (j + F[x]);                                                                      \
+      P = fma_(K.v1f, p, fma_(K.v2, q, e));                                                         \
+      Q = fma_(K.v1f, q, fma_(K.v2, p, e));                                                         \
+      T = fma_(K.z1f, T, fma_(K.z2, p + q, fma_(K.zjf, j, R(1.0 / 72.0) * F[x])));                   \
+    }
+    LBMK_VEC(LBMK_R(1, 0, 0), LBMK_R(1, 2, 0), LBMK_R(1, 0, 2), LBMK_R(1, 2, 2), 0)
+    LBMK_VEC(LBMK_R(0, 1, 0), LBMK_R(0, 1, 2), LBMK_R(2, 1, 0), LBMK_R(2, 1, 2), 1)
+    LBMK_VEC(LBMK_R(0, 0, 1), LBMK_R(2, 0, 1), LBMK_R(0, 2, 1), LBMK_R(2, 2, 1), 2)
 #undef LBMK_VEC
+  } else {
+    const R hs = R(-0.5) * s_sh;
+    const R L = fma_(fma_(R(1.0 / 6.0), s_sh, -K.s5h), S2, R(-0.5) * m_abs);
+    LBMK_R(2, 0, 0) = fma_(R(0.5), LBMK_R(2, 0, 0), fma_(hs, h0, fma_(R(0.5), pi0, L)));
+    LBMK_R(0, 2, 0) = fma_(R(0.5), LBMK_R(0, 2, 0), fma_(hs, h1, fma_(R(0.5), pi1, L)));
+    LBMK_R(0, 0, 2) = fma_(R(0.5), LBMK_R(0, 0, 2), fma_(hs, h2, fma_(R(0.5), pi2, L)));
+    const R CQ = fma_(a2, S2, fma_(K.q4, S4, R(1.0 / 12.0) * Z));
+    const R E3 = R(1.0 / 3.0) * Btr;                                       // equilibrium of <b^2c^2>: E3 - sg_a/3
+#define LBMK_EVEN(Q, h2a, sg, pi)                                                                   \
+    {                                                                                                 \
+      const R hq = Q - fma_(R(-1.0 / 3.0), sg, E3);                                                   \
+      Q = fma_(R(0.25), Q, fma_(K.q1, hq, fma_(b, h2a, fma_(R(-1.0 / 12.0), pi, CQ))));               \
+    }
+    LBMK_EVEN(LBMK_R(0, 2, 2), h0, sg0, pi0)
+    LBMK_EVEN(LBMK_R(2, 0, 2), h1, sg1, pi1)
+    LBMK_EVEN(LBMK_R(2, 2, 0), h2, sg2, pi2)
+#undef LBMK_EVEN
+    {
+      const R ht = fma_(R(-1.0 / 3.0), E3, LBMK_R(2, 2, 2));
+      LBMK_R(2, 2, 2) = fma_(R(0.125), LBMK_R(2, 2, 2),
+                             fma_(K.t1, ht, fma_(K.t4, S4, fma_(K.t2, S2, R(1.0 / 72.0) * Z))));
+    }
+    // pairs <ab>, <abc^2>
+    const R c4 = R(0.5) * hs, k = fma_(R(-1.0 / 12.0), s_sh, K.pk);        // -s/4, (s21 - s)/12
+#define LBMK_PAIR(P, Q, x, y)                                                                       \
+    {                                                                                                 \
+      const R t = fma_(u[x], w[y], u[y] * w[x]);                                                      \
+      const R g = fma_(m[x], n[y], fma_(u[x], F[y], u[y] * F[x]));                                    \
+      const R h = fma_(R(-0.5), t, P);                                                                \
+      P = fma_(R(0.25), P, fma_(c4, h, R(0.25) * g));                                                 \
+      const R hq = fma_(R(-1.0 / 6.0), t, Q);                                                         \
+      Q = fma_(R(0.125), Q, fma_(K.p1, hq, fma_(k, h, R(1.0 / 24.0) * g)));                           \
+    }
+    LBMK_PAIR(LBMK_R(1, 1, 0), LBMK_R(1, 1, 2), 0, 1)
+    LBMK_PAIR(LBMK_R(0, 1, 1), LBMK_R(2, 1, 1), 1, 2)
+    LBMK_PAIR(LBMK_R(1, 0, 1), LBMK_R(1, 2, 1), 0, 2)
+#undef LBMK_PAIR
+    // vectors <a>, <ab^2>, <ac^2>, <ab^2c^2>
+#define LBMK_VEC(J, P, Q, T, x)                                                                     \
+    {                                                                                                 \
+      const R j3 = R(1.0 / 3.0) * J, F12 = R(1.0 / 12.0) * F[x], hp = P - j3, hq = Q - j3;            \
+      P = fma_(R(0.25), P, fma_(K.v1, hp, fma_(K.v2, hq, F12)));                                      \
+      Q = fma_(R(0.25), Q, fma_(K.v1, hq, fma_(K.v2, hp, F12)));                                      \
+      const R ht = fma_(R(-1.0 / 3.0), j3, T);                                                        \
+      T = fma_(R(0.125), T, fma_(K.z1, ht, fma_(K.z2, hp + hq, R(1.0 / 72.0) * F[x])));               \
+      J = R(0.5) * (J + F[x]);                                                                        \
+    }
+    LBMK_VEC(LBMK_R(1, 0, 0), LBMK_R(1, 2, 0), LBMK_R(1, 0, 2), LBMK_R(1, 2, 2), 0)
+    LBMK_VEC(LBMK_R(0, 1, 0), LBMK_R(0, 1, 2), LBMK_R(2, 1, 0), LBMK_R(2, 1, 2), 1)
+    LBMK_VEC(LBMK_R(0, 0, 1), LBMK_R(2, 0, 1), LBMK_R(0, 2, 1), LBMK_R(2, 2, 1), 2)
+#undef LBMK_VEC
+  }
   LBMK_R(1, 1, 1) = K.d1 * LBMK_R(1, 1, 1);
 }
 

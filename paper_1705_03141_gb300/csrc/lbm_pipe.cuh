@@ -195,7 +195,7 @@ __global__ void __launch_bounds__(TP_THREADS, TP_MINB)
     if (lane == 0) mbar_arrive(&empty[s]);  // the populations and gradients are in registers
     if (act && ok) {
       float f[27];
-      const Recol<float> rc = collide(K, rho_r, ft, gphi, grho, f);
+      const Recol<float> rc = collide<true>(K, rho_r, ft, gphi, grho, f);
       const bool recol = __any_sync(__activemask(), any_(rc.has_n));
       NodeMap nm;
       AoRow ar;

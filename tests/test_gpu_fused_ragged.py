@@ -1,0 +1,60 @@
+"""The fused density pass on rows that do not fill whole 32-node blocks, against the two-pass scheme.
+
+Both compute one update; what differs is the rounding of the densities that enter the gradients: the
+fused pass sums them in fixed point (2^-25 for densities up to 1), the density pass in FP32 (2^-24 of
+each partial sum).  One step therefore changes the fields by a few 2^-24 of the density; 40 steps
+of a smooth, stable flow let that grow to at most the bound on FP32 against the oracle
+(2e-5 of the density scale, 1e-4 of max|u| + 3e-6, tests/test_gpu_parity.py).
+"""
+import numpy as np
+import pytest
+
+import lbm_inputs as L
+import paper_1705_03141_gb300 as pkg
+
+pytestmark = pytest.mark.gpu
+
+# last block with 1, 2 and 31 nodes, less than one block, whole blocks; every x face that has fast rows
+SHAPES = [(33, 8, 9), (34, 9, 8), (63, 7, 10), (21, 12, 9), (64, 8, 8)]
+FACES = {"periodic": (0, 0, 0, 0, 0, 0), "jet": (2, 2, 2, 2, 3, 4), "walls": (2, 2, 1, 1, 1, 1)}
+
+
+def _work(shape, faces):
+    p = dict(L.parity_cases()[3][1]["params"])
+    p.update(bc=FACES[faces])
+    p["inflow"] = dict(p["inflow"], xc=0.5 * (shape[0] - 1), yc=0.5 * (shape[1] - 1), D=4.0) if faces == "jet" else None
+    return dict(name=faces, shape=shape, params=p, fields=("random_blobs", dict(seed=9, blobs=3)), steps=40)
+
+
+def _run(w, variant, block=0):
+    rr, rb, u = L.initial_fields(w, seed=2, u_amp=0.02)
+    lat = pkg.Lattice(w["shape"], w["params"], storage="f32", variant=variant, block=block)
+    lat.init_fields(rr, rb, u)
+    for n in (1, 23, 16):
+        lat.step(n)
+    out = lat.macro()
+    lat.synchronize()
+    lat.close()
+    return out
+
+
+@pytest.mark.parametrize("faces", list(FACES))
+@pytest.mark.parametrize("shape", SHAPES)
+def test_fused_ragged_rows(cuda, shape, faces):
+    w = _work(shape, faces)
+    ar, ab, au = _run(w, 1)
+    scale = max(np.max(ar), np.max(ab))
+    for block in (1, 2, 3):
+        r, b, u = _run(w, 3, block)
+        assert np.max(np.abs(r - ar)) < 2e-5 * scale and np.max(np.abs(b - ab)) < 2e-5 * scale
+        assert np.max(np.abs(u - au)) < 1e-4 * np.max(np.abs(au)) + 3e-6
+    again = _run(w, 3, 2)
+    for x, y in zip(again, _run(w, 3, 2)):
+        assert np.array_equal(x, y)  # bitwise reproducible
+
+
+def test_library_choice_by_size(cuda):
+    for shape, variant in (((64, 20, 40), 3), ((66, 20, 40), 1), ((126, 104, 81), 3)):
+        lat = pkg.Lattice(shape, _work(shape, "periodic")["params"], storage="f32")
+        assert lat.variant == variant
+        lat.close()
