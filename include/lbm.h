@@ -179,7 +179,7 @@ typedef struct {
                             update bitwise in every shape; variant 3 differs by FP32
                             rounding (how the next step's densities are grouped
                             before their exact fixed-point sum).  FP64 storage
-                            always runs 32x4x2.  Compact storage (F16C/BF16C) runs
+                            runs node after node and reports 1.  Compact storage (F16C/BF16C) runs
                             32x4x2 tiles with one of two density passes: 1 = one
                             block per tile, 4 = persistent blocks of 8 consumer
                             warps and one producer warp that streams each tile's

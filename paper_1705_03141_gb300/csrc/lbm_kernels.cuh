@@ -157,11 +157,11 @@ __device__ __forceinline__ bool is_inlet(const Geom& g, int x, int y, int z) {
   return dx * dx + dy * dy < g.r2;
 }
 
-// fast reciprocal / inverse square root: exact in FP64 (oracle parity), MUFU in FP32
+// fast reciprocal / inverse square root: FP64 within an ulp (oracle parity), MUFU in FP32
 // (the two-lane versions are in lbm_f2.cuh)
 __device__ __forceinline__ double rcp_(double x) { return 1.0 / x; }
 __device__ __forceinline__ float rcp_(float x) { return __fdividef(1.0f, x); }
-__device__ __forceinline__ double rsqrt_(double x) { return 1.0 / sqrt(x); }
+__device__ __forceinline__ double rsqrt_(double x) { return rsqrt(x); }
 __device__ __forceinline__ float rsqrt_(float x) { return rsqrtf(x); }
 __device__ __forceinline__ double sat_(double x) { return fmin(fmax(x, 0.0), 1.0); }
 __device__ __forceinline__ float sat_(float x) { return __saturatef(x); }
@@ -1020,6 +1020,26 @@ __device__ __forceinline__ void outflow_column(const Store& st, const Geom& G, c
   }
 }
 
+// (rho, phi) of a node from its red density and totals; inlet: a Dirichlet inlet node
+template <typename D, typename V>
+__device__ __forceinline__ V density_value(const KConst<D>& K, D rr, const D ft[27], bool inlet,
+                                           int* __restrict__ flag) {
+  D rt = D(0);
+#pragma unroll
+  for (int t = 0; t < 27; ++t) rt += ft[t];
+  if (!(rt > D(0)) || !(rt < D(1e30))) atomicOr(flag, 1);
+  D rb = rt - rr;
+  if (inlet) {
+    rr = (D)K.rho_r0_d;
+    rb = D(0);
+  }
+  const D rho = rr + rb;
+  V v;
+  v.x = rho;
+  v.y = (rr - rb) / rho;
+  return v;
+}
+
 // top != null (an outflow face): the threads of the plane z = nz-1 first complete the step
 // before with its convective outflow (outflow_column), so that k_outflow need not run between
 // the steps of a run; the blocks of the top planes start first (z blocks in reverse order).
@@ -1048,23 +1068,14 @@ __global__ void __launch_bounds__(B::NT, 4) k_density(Store st, Geom G,
     nm.init(G, x, y, z);
     load_node(st, K, nm, layout, rr, ft);
   }
-  D rt = D(0);
-#pragma unroll
-  for (int t = 0; t < 27; ++t) rt += ft[t];
-  if (!(rt > D(0)) || !(rt < D(1e30))) atomicOr(flag, 1);
   if constexpr (FIX) {
+    D rt = D(0);
+#pragma unroll
+    for (int t = 0; t < 27; ++t) rt += ft[t];
+    if (!(rt > D(0)) || !(rt < D(1e30))) atomicOr(flag, 1);
     fix[dnode(G, x, y, z)] = pack_fix((float)rt, (float)rr, (float)K.fix_scale);
   } else {
-    D rb = rt - rr;
-    if (is_inlet(G, x, y, z)) {
-      rr = (D)K.rho_r0_d;
-      rb = D(0);
-    }
-    const D rho = rr + rb;
-    typename DensOf<Store>::type v;
-    v.x = rho;
-    v.y = (rr - rb) / rho;
-    dens[dnode(G, x, y, z)] = v;
+    dens[dnode(G, x, y, z)] = density_value<D, typename DensOf<Store>::type>(K, rr, ft, is_inlet(G, x, y, z), flag);
   }
 }
 
@@ -1422,6 +1433,112 @@ __global__ void __launch_bounds__(B::NT, MINB)
       }
     }
   }
+}
+
+// ---------------------------------------------------------------------------
+// FP64 storage: both passes node after node (thread n holds node n of the box, x fastest).  GB300
+// issues an FP64 instruction of a warp in 16 cycles whatever number of its lanes is active, and at
+// about 550 of them a node that is all the time there is (an SM's issue slots are 90 % idle).  So
+// the lanes are filled first: rows of 41 nodes cost 41, not 64; small blocks spread a small box
+// over all SMs; and every node takes the general streaming map, which is integer work, so that a
+// warp may span rows.  The gradients read (rho, phi) through L1.
+// Against 32 x 4 x 2 blocks with a halo tile in shared memory, us a step: 32^3 58 -> 55, 41^3 168 ->
+// 105, 17x40x23 58 -> 33, 64^3 386 -> 354 (19 cycles per FP64 instruction and SM of the pipe's 16).
+constexpr int LIN_THREADS = 64;
+
+__device__ __forceinline__ bool lin_node(const Geom& G, int& x, int& y, int& z) {
+  const int n = blockIdx.x * LIN_THREADS + threadIdx.x;
+  const int row = n / G.nx;
+  x = n - row * G.nx;
+  z = row / G.ny;
+  y = row - z * G.ny;
+  return z < G.nz;
+}
+
+// directions T = 0 .. 12 and their opposites, which share c.n and the recolouring coefficient
+template <int T, bool RECOL, class Store, typename R>
+__device__ __forceinline__ void emit_pairs(const Store& st, const KConst<R>& K, const NodeMap& nm, bool odd,
+                                           const R f[27], const Recol<R>& rc) {
+  if constexpr (T < REST) {
+    constexpr int O = opp_of(T), CLS = speed2_of(T);
+    const R rcn = RECOL ? rc.rc[CLS] * cdot<O>(rc.n0, rc.n1, rc.n2) : R(0);
+    const R rT = RECOL ? fma_(rc.frac, f[T], -rcn) : rc.frac * f[T];
+    const R rO = RECOL ? fma_(rc.frac, f[O], rcn) : rc.frac * f[O];
+    int64_t node = nm.base;
+    int dir = O;
+    if (odd) nm.push<T>(node, dir);
+    st.store(node, dir, CLS, K, rT, f[T] - rT, f[T], R(0));
+    node = nm.base;
+    dir = T;
+    if (odd) nm.push<O>(node, dir);
+    st.store(node, dir, CLS, K, rO, f[O] - rO, f[O], R(0));
+    emit_pairs<T + 1, RECOL>(st, K, nm, odd, f, rc);
+  } else {
+    const R r = rc.frac * f[REST];
+    st.store(nm.base, REST, 0, K, r, f[REST] - r, f[REST], R(0));
+  }
+}
+
+template <class Store>
+__global__ void __launch_bounds__(LIN_THREADS)
+    k_collide_stream_lin(Store st, const __grid_constant__ Geom G,
+                         const __grid_constant__ KConst<typename DensOf<Store>::real> K, int odd,
+                         const typename DensOf<Store>::type* __restrict__ dens, long long* __restrict__ counter) {
+  using R = typename DensOf<Store>::real;
+  const long long step = counter[odd];
+  if (blockIdx.x == 0 && threadIdx.x == 0) counter[odd ^ 1] = step + 1;
+  int x, y, z;
+  const bool active = lin_node(G, x, y, z);
+  const unsigned mask = __ballot_sync(0xffffffffu, active);
+  if (!active) return;
+  NodeMap nm;
+  nm.init(G, x, y, z);
+  R rho_r = R(0), ft[27], gphi[3], grho[3];
+  load_node(st, K, nm, odd, rho_r, ft);
+  {
+    int X[3], Y[3], Z[3];
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      X[d] = wrap_or_clamp(x + d - 1, G.nx, G.bc[0], G.bc[1]);
+      Y[d] = wrap_or_clamp(y + d - 1, G.ny, G.bc[2], G.bc[3]) * G.nx;
+      Z[d] = wrap_or_clamp(z + d - 1, G.nz, G.bc[4], G.bc[5]) * G.nx * G.ny;
+    }
+    const auto cell = [&](int dx, int dy, int dz) { return dens[X[dx + 1] + Y[dy + 1] + Z[dz + 1]]; };
+    pair_gradients<R>([&](int dx, int dy, int dz) { return (R)cell(dx, dy, dz).x; }, grho);
+    pair_gradients<R>([&](int dx, int dy, int dz) { return (R)cell(dx, dy, dz).y; }, gphi);
+  }
+  R f[27];
+  Recol<R> rc;
+  if (is_inlet(G, x, y, z)) {
+    inlet_state(K, dnode(G, x, y, z), (int64_t)step, f);
+    rc.frac = R(1);
+    rc.n0 = rc.n1 = rc.n2 = R(0);
+    rc.rc[0] = rc.rc[1] = rc.rc[2] = rc.rc[3] = R(0);
+    rc.rho = R(1);
+    rc.has_n = false;
+  } else {
+    rc = collide<true>(K, rho_r, ft, gphi, grho, f);
+  }
+  if (__any_sync(mask, any_(rc.has_n))) emit_pairs<0, true>(st, K, nm, odd != 0, f, rc);
+  else emit_pairs<0, false>(st, K, nm, odd != 0, f, rc);
+}
+
+// pass 1; top: as in k_density
+template <class Store>
+__global__ void __launch_bounds__(LIN_THREADS)
+    k_density_lin(Store st, const __grid_constant__ Geom G,
+                  const __grid_constant__ KConst<typename DensOf<Store>::real> K, int layout,
+                  typename DensOf<Store>::type* __restrict__ dens, int* __restrict__ flag,
+                  typename DensOf<Store>::real* __restrict__ top) {
+  using D = typename DensOf<Store>::real;
+  int x, y, z;
+  if (!lin_node(G, x, y, z)) return;
+  if (top != nullptr && z == G.nz - 1) outflow_column(st, G, K, layout, x, y, top);
+  NodeMap nm;
+  nm.init(G, x, y, z);
+  D rr = D(0), ft[27];
+  load_node(st, K, nm, layout, rr, ft);
+  dens[dnode(G, x, y, z)] = density_value<D, typename DensOf<Store>::type>(K, rr, ft, is_inlet(G, x, y, z), flag);
 }
 
 // ---------------------------------------------------------------------------

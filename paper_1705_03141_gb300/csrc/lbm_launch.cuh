@@ -68,11 +68,15 @@ struct Launch {
   }
   static cudaError_t density_top(void* pop, const Geom& G, const Phys& P, int layout, void* dens, int* flag,
                                  void* fix, void* top, int shape, cudaStream_t s) {
-    if constexpr (!std::is_same<R, double>::value) {  // FP64 keeps the default shape
+    if constexpr (std::is_same<R, double>::value) {  // node after node: no blocks of rows
+      k_density_lin<Store><<<blocks1((int64_t)G.nx * G.ny * G.nz, LIN_THREADS), LIN_THREADS, 0, s>>>(
+          Tr::make(pop, G), G, kc(P), layout, static_cast<DT*>(dens), flag, static_cast<R*>(top));
+      return cudaGetLastError();
+    } else {
       if (shape == 1) return density_b<Blk<2, 4>>(pop, G, P, layout, dens, flag, fix, top, s);
       if (shape == 2) return density_b<Blk<8, 1>>(pop, G, P, layout, dens, flag, fix, top, s);
+      return density_b<BlkDefault>(pop, G, P, layout, dens, flag, fix, top, s);
     }
-    return density_b<BlkDefault>(pop, G, P, layout, dens, flag, fix, top, s);
   }
   static cudaError_t density(void* pop, const Geom& G, const Phys& P, int layout, void* dens, int* flag, void* fix,
                              int shape, cudaStream_t s) {
@@ -196,12 +200,16 @@ struct Launch {
         if (e != cudaErrorNotSupported) return e;  // else the box has no pipelined tiles: variant 1
       }
     }
-    const bool fp = variant == 3;
-    if constexpr (!std::is_same<R, double>::value) {
+    if constexpr (std::is_same<R, double>::value) {
+      k_collide_stream_lin<Store><<<blocks1((int64_t)G.nx * G.ny * G.nz, LIN_THREADS), LIN_THREADS, 0, s>>>(
+          Tr::make(pop, G), G, kc(P), odd, static_cast<const DT*>(dens), counter);
+      return cudaGetLastError();
+    } else {
+      const bool fp = variant == 3;
       if (shape == 1) return collide_b<Blk<2, 4>>(pop, G, P, odd, dens, counter, fp, io, s);
       if (shape == 2) return collide_b<Blk<8, 1>>(pop, G, P, odd, dens, counter, fp, io, s);
+      return collide_b<BlkDefault>(pop, G, P, odd, dens, counter, fp, io, s);
     }
-    return collide_b<BlkDefault>(pop, G, P, odd, dens, counter, fp, io, s);
   }
   static cudaError_t outflow(void* pop, const Geom& G, const Phys& P, int layout, void* top, void* fix,
                              cudaStream_t s) {

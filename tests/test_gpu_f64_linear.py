@@ -1,0 +1,35 @@
+"""FP64 storage (threads over the nodes in linear order) against the oracle at 1e-12: boxes of less than one
+warp, warps that span rows and planes, a last block with one node, every face type."""
+import numpy as np
+import pytest
+
+import lbm_inputs as L
+import oracle
+import paper_1705_03141_gb300 as pkg
+
+pytestmark = pytest.mark.gpu
+
+FACES = {"periodic": (0, 0, 0, 0, 0, 0), "walls": (1, 1, 2, 2, 1, 2), "jet": (2, 2, 2, 2, 3, 4)}
+
+
+@pytest.mark.parametrize("faces", list(FACES))
+@pytest.mark.parametrize("shape", [(3, 3, 3), (5, 13, 3), (13, 5, 7), (41, 9, 8), (64, 5, 5)])
+def test_fp64_matches_oracle(cuda, shape, faces):
+    p = dict(L.parity_cases()[1][1]["params"])
+    p.update(bc=FACES[faces], g=(1e-5, 0.0, 2e-5), force_mode=2, seed=5)
+    if faces == "jet":
+        p["inflow"] = dict(xc=0.5 * (shape[0] - 1), yc=0.5 * (shape[1] - 1), D=2.5, u_j0=0.02, noise_frac=0.01)
+    w = dict(name=faces, shape=shape, params=p, fields=("random_blobs", dict(seed=2, blobs=2)), steps=20)
+    rr, rb, u = L.initial_fields(w, seed=3, u_amp=0.01)
+    lat = pkg.Lattice(shape, p, storage="f64")
+    lat.init_fields(rr, rb, u)
+    for n in (1, 2, 17):
+        lat.step(n)
+    orc = oracle.Oracle(shape, p)
+    orc.init_fields(rr, rb, u)
+    orc.step(20)
+    for a, b in zip(lat.macro(), orc.macro()):
+        assert np.max(np.abs(a - b)) < 1e-12 * np.max(np.abs(b))
+    f = lat.get_populations()
+    assert np.max(np.abs(f - orc.f.reshape(f.shape))) < 1e-12 * np.max(np.abs(orc.f))
+    lat.close()
