@@ -69,7 +69,7 @@ struct CompactStore {
     __stcs(A + e0 + dir * 32, float_to_dev(f - K.refB[cls]));
   }
   // by a node's base pointer p1 = A + e1 and a 32-bit element offset (fast rows)
-  __device__ __forceinline__ float load_rel(const uint16_t* p1, int rel, int dir, int cls,
+  __device__ __forceinline__ float load_rel(const uint16_t* p1, int64_t rel, int dir, int cls,
                                             const KConst<float>& K) const {
     if (dir == REST) {
       const uint32_t hi = __ldcs(p1 + (rel + REST_HI * 32)), lo = __ldcs(p1 + (rel + REST_LO * 32));
@@ -77,7 +77,7 @@ struct CompactStore {
     }
     return K.refB[cls] + dev_to_float(__ldcs(p1 + (rel + dir * 32)));
   }
-  __device__ __forceinline__ void store_rel(uint16_t* p1, int rel, int dir, int cls, const KConst<float>& K,
+  __device__ __forceinline__ void store_rel(uint16_t* p1, int64_t rel, int dir, int cls, const KConst<float>& K,
                                             float f) const {
     if (dir == REST) {
       const uint32_t b = __float_as_uint(f);
@@ -135,15 +135,15 @@ __device__ __forceinline__ void fast_totals(const CompactStore<BF16>& st, const 
   const uint16_t* p1 = st.A + ar.e[1];
 #pragma unroll
   for (int t = 0; t < 27; ++t) {
-    int rel = 0;
+    int64_t rel = 0;
     if (LAYOUT) {
       switch (26 - t) {
-#define LBMK_CASE(k) case k: rel = ar.rel0<k, CPLANES>(G); break;
+#define LBMK_CASE(k) case k: rel = ar.rel0<k>(); break;
         LBMK_CASE(0) LBMK_CASE(1) LBMK_CASE(2) LBMK_CASE(3) LBMK_CASE(4) LBMK_CASE(5) LBMK_CASE(6)
         LBMK_CASE(7) LBMK_CASE(8) LBMK_CASE(9) LBMK_CASE(10) LBMK_CASE(11) LBMK_CASE(12) LBMK_CASE(13)
         LBMK_CASE(14) LBMK_CASE(15) LBMK_CASE(16) LBMK_CASE(17) LBMK_CASE(18) LBMK_CASE(19) LBMK_CASE(20)
         LBMK_CASE(21) LBMK_CASE(22) LBMK_CASE(23) LBMK_CASE(24) LBMK_CASE(25)
-        default: rel = ar.rel0<26, CPLANES>(G); break;
+        default: rel = ar.rel0<26>(); break;
 #undef LBMK_CASE
       }
     }
@@ -209,11 +209,12 @@ __global__ void __launch_bounds__(NTHREADS, 3) k_density_c(CompactStore<BF16> st
                                                            const __grid_constant__ KConst<float> K, int layout,
                                                            float2* __restrict__ dens, int* __restrict__ flag) {
   __shared__ float4 rt[TILE];
-  const int x0 = blockIdx.x * BX, y0 = blockIdx.y * BY, z0 = blockIdx.z * BZ;
+  const int x0 = blockIdx.x * BX, y0 = blockIdx.y * BY;
+  const int z0 = face_first(blockIdx.z, gridDim.z, BC_NOSLIP) * BZ;  // all face rows take the general path
   const int x = x0 + threadIdx.x, y = y0 + threadIdx.y, z = z0 + threadIdx.z;
   const int tid = threadIdx.x + BX * (threadIdx.y + BY * threadIdx.z);
   const bool top = on_top(G, z);
-  const bool fast = !top && fast_row(G, y, z);
+  const bool fast = !top && interior_row(G, y, z);
   const bool active = x < G.nx && y < G.ny && z < G.nz;
   float f[27];
   if (active && !top) {
@@ -485,7 +486,7 @@ __global__ void __launch_bounds__(NG * NTHREADS + 32, MINB)
       if (lane < TX - 32) red |= __float_as_uint(rr[32 + lane].x);
     }
     const bool blue = !__any_sync(0xffffffffu, (red << 1) != 0u);
-    if (x < G.nx && y < G.ny && z < G.nz && !on_top(G, z) && fast_row(G, y, z)) {
+    if (x < G.nx && y < G.ny && z < G.nz && !on_top(G, z) && interior_row(G, y, z)) {
       // mirror x faces: the face lane's emitter beyond the face is the face node itself
       const bool mlo = x == 0, mhi = x == G.nx - 1;
       float f[27];
@@ -574,7 +575,7 @@ __global__ void __launch_bounds__(NTHREADS, 4)
     k_collide_stream_c(CompactStore<BF16> st, const __grid_constant__ Geom G, const __grid_constant__ KConst<float> K,
                        int odd, const float2* __restrict__ dens, long long* __restrict__ counter) {
   __shared__ float2 tile[TILE];
-  const int x0 = blockIdx.x * BX, y0 = blockIdx.y * BY, z0 = blockIdx.z * BZ;
+  const int x0 = blockIdx.x * BX, y0 = blockIdx.y * BY, z0 = face_first(blockIdx.z, gridDim.z, G.bc[5]) * BZ;
   const int x = x0 + threadIdx.x, y = y0 + threadIdx.y, z = z0 + threadIdx.z;
   const bool active = x < G.nx && y < G.ny && z < G.nz;
   const int tid = threadIdx.x + BX * (threadIdx.y + BY * threadIdx.z);
@@ -668,14 +669,14 @@ __global__ void __launch_bounds__(NTHREADS, 4)
     } else {
 #pragma unroll
       for (int t = 0; t < 27; ++t) {
-        int rel;
+        int64_t rel;
         switch (t) {
-#define LBMK_CASE(k) case k: rel = ar.rel0<k, CPLANES>(G); break;
+#define LBMK_CASE(k) case k: rel = ar.rel0<k>(); break;
           LBMK_CASE(0) LBMK_CASE(1) LBMK_CASE(2) LBMK_CASE(3) LBMK_CASE(4) LBMK_CASE(5) LBMK_CASE(6)
           LBMK_CASE(7) LBMK_CASE(8) LBMK_CASE(9) LBMK_CASE(10) LBMK_CASE(11) LBMK_CASE(12) LBMK_CASE(13)
           LBMK_CASE(14) LBMK_CASE(15) LBMK_CASE(16) LBMK_CASE(17) LBMK_CASE(18) LBMK_CASE(19) LBMK_CASE(20)
           LBMK_CASE(21) LBMK_CASE(22) LBMK_CASE(23) LBMK_CASE(24) LBMK_CASE(25)
-          default: rel = ar.rel0<26, CPLANES>(G); break;
+          default: rel = ar.rel0<26>(); break;
 #undef LBMK_CASE
         }
         st.store_rel(p1, rel, t, speed2_of(t), K, f[t]);

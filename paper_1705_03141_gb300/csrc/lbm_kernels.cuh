@@ -227,20 +227,25 @@ struct NodeMap {
   }
 };
 
-// Streaming map of a node on a "fast row": its y and z neighbours are inside the
-// box (a warp is one x-row of a block, so this is warp-uniform) and neither x
-// face bounces back.  Storage rows are padded to a multiple of 32 nodes (nxs),
-// so a y/z shift moves whole 32-node storage blocks, and S(x, t) only needs the
-// element index of plane 0 of the x-shifted node, e[c_x + 1]; a specular
-// reflection at an x face turns every direction with that c_x into the one two
-// planes away, so it is folded into e as a constant plane shift.  (Lanes past
-// nx in the last block of a row are idle; their padding slots are never used.)
+// Streaming map of a node on a "fast row": no face the row touches bounces back (a warp is one x-row
+// of a block, so this is warp-uniform).  Storage rows are padded to a multiple of 32 nodes (nxs),
+// so a y/z shift moves whole 32-node storage blocks, across a periodic face too, and S(x, t) only
+// needs the offset of the row (y + c_y, z + c_z) and the element index of plane 0 of the x-shifted node; a
+// specular reflection at a face keeps the coordinate and turns every direction with that component into
+// the one 2 (x), 6 (y) or 18 (z) planes away, so it is folded into the shift as a constant number of
+// planes.  (Lanes past nx in the last block of a row are idle; their padding slots are never used.)
+// Only bouncing rows take the general map (NodeMap), about four times the instructions of a step.  Against
+// all face rows on it (12 % of a 32^3 box, 4 % of a 96x96x384 one), us a step: 32^3 f16 13.1 -> 8.5, f32
+// 15.7 -> 8.7; 64^3 f16 24.0 -> 21.6, f32 32.6 -> 27.0, c16 33.9 -> 29.4; 80x80x320 jet f16 152 -> 149,
+// c16 180 -> 175; 128x128x512 jet f16 495 -> 490.
 struct AoRow {
   int64_t e[3];
-  int dxm, dxp;  // e[0] - e[1] and e[2] - e[1]
+  int dxm, dxp;        // e[0] - e[1] and e[2] - e[1]
+  int ym, yp, zm, zp;  // row shifts in units of 32 elements (|shift| < 2^31: NodeMap keeps the box below 2^31 nodes)
   // the node's storage block (x >> 5) + (nxs / 32)(y + ny (z + 1)) fits 32 bits; within a block the
-  // x neighbours are one element away, across a block edge one block of PLANES planes minus 31
-  template <int PLANES>
+  // x neighbours are one element away, across a block edge one block of PLANES planes minus 31.
+  // INTERIOR: the row touches no y or z face
+  template <int PLANES, bool INTERIOR = false>
   __device__ __forceinline__ void init(const Geom& g, int x, int y, int z) {
     const int lane = x & 31;
     const int b = (x >> 5) + (g.nxs >> 5) * (y + g.ny * (z + 1));
@@ -252,33 +257,49 @@ struct AoRow {
     if (x == g.nx - 1) dxp = g.bc[1] == BC_PERIODIC ? (int)(elem_index(snode(g, 0, y, z), PLANES, 0) - e[1]) : -2 * 32;
     e[0] = e[1] + dxm;
     e[2] = e[1] + dxp;
+    const int sy = (g.nxs >> 5) * PLANES, sz = sy * g.ny;
+    ym = -sy;
+    yp = sy;
+    zm = -sz;
+    zp = sz;
+    if (!INTERIOR) {  // an outflow or halo face: the ghost plane, as inside the box
+      if (y == 0) ym = g.bc[2] == BC_PERIODIC ? sz - sy : 6;
+      if (y == g.ny - 1) yp = g.bc[3] == BC_PERIODIC ? sy - sz : -6;
+      if (z == 0 && g.bc[4] != BC_HALO) zm = g.bc[4] == BC_PERIODIC ? (g.nz - 1) * sz : 18;
+      if (z == g.nz - 1 && g.bc[5] != BC_HALO && g.bc[5] != BC_OUTFLOW)
+        zp = g.bc[5] == BC_PERIODIC ? -(g.nz - 1) * sz : -18;
+    }
   }
-  // element offset of the storage row (y + cy, z + cz) from the node's own row (a grid-wide value)
-  template <int PLANES>
-  __device__ __forceinline__ int row_off(const Geom& g, int cy, int cz) const {
-    return cy * (g.nxs * PLANES) + cz * (g.nxs * g.ny * PLANES);
+  // element offset of the storage row that (c_y, c_z) leads to from the node's own row
+  __device__ __forceinline__ int64_t row(int cy, int cz) const {
+    return (int64_t)((cy < 0 ? ym : (cy > 0 ? yp : 0)) + (cz < 0 ? zm : (cz > 0 ? zp : 0))) * 32;
   }
-  // element offset of plane 0 of the slot S(x, t) from the node's own plane 0, in 32 bits (a z
-  // plane of storage holds fewer than 2^31 elements, checked at creation): slot pointers are the
-  // node's base pointer plus one 32-bit offset, one wide multiply-add per access.  nxs is a
-  // multiple of 32, so a y step moves nxs / 32 whole blocks of PLANES * 32 elements: nxs * PLANES
-  // elements (a z step nxs * ny * PLANES), products the whole grid shares.
-  template <int T, int PLANES>
-  __device__ __forceinline__ int rel0(const Geom& g) const {
-    const int dx = cx_of(T) < 0 ? dxm : (cx_of(T) > 0 ? dxp : 0);
-    return dx + cy_of(T) * (g.nxs * PLANES) + cz_of(T) * (g.nxs * g.ny * PLANES);
-  }
-  // element index of plane 0 of the slot S(x, t) (add the plane of t)
-  template <int T, int PLANES>
-  __device__ __forceinline__ int64_t slot0(const Geom& g) const {
-    return e[cx_of(T) + 1] + (int64_t)(cy_of(T) * (g.nxs * PLANES) + cz_of(T) * (g.nxs * g.ny * PLANES));
+  // element offset of plane 0 of the slot S(x, t) from the node's own plane 0 (add the plane of t)
+  template <int T>
+  __device__ __forceinline__ int64_t rel0() const {
+    return row(cy_of(T), cz_of(T)) + (cx_of(T) < 0 ? dxm : (cx_of(T) > 0 ? dxp : 0));
   }
 };
 
+// rows whose streaming map is AoRow's
 __device__ __forceinline__ bool fast_row(const Geom& g, int y, int z) {
+  return g.bc[0] != BC_NOSLIP && g.bc[1] != BC_NOSLIP && (y > 0 || g.bc[2] != BC_NOSLIP) &&
+         (y < g.ny - 1 || g.bc[3] != BC_NOSLIP) && (z > 0 || g.bc[4] != BC_NOSLIP) &&
+         (z < g.nz - 1 || g.bc[5] != BC_NOSLIP);
+}
+// fast rows that touch no y or z face
+__device__ __forceinline__ bool interior_row(const Geom& g, int y, int z) {
   return y > 0 && y < g.ny - 1 && z > 0 && z < g.nz - 1 && g.bc[0] != BC_NOSLIP && g.bc[1] != BC_NOSLIP;
 }
 
+
+// Layer of blocks number i of n to start, where the last layer lies at a face of condition bc: a
+// no-slip face comes second instead of last, since the general map of its rows, used nowhere
+// else, is not in the instruction cache by then and would be the pass's tail (64x64x256
+// f16 with no-slip z faces 78.4 -> 74.5 us a step, f32 109 -> 101; 32x32x128 f16 17.9 -> 14.2).
+__device__ __forceinline__ int face_first(int i, int n, int bc) {
+  return bc != BC_NOSLIP || i == 0 ? i : (i == 1 ? n - 1 : i - 1);
+}
 
 // slot holding the post-streaming population (x, t) in a layout (runtime t)
 __device__ __forceinline__ void slot_of(const NodeMap& nm, int layout, int t, int64_t& node, int& dir) {
@@ -579,7 +600,7 @@ __device__ __forceinline__ void load_node_fast(const Store& st, const KConst<R>&
     // ascending order, as on even steps)
 #pragma unroll
     for (int g9 = 8; g9 >= 0; --g9) {
-      const auto* rp = p1 + ar.template row_off<Store::PLANES>(G, g9 % 3 - 1, g9 / 3 - 1);
+      const auto* rp = p1 + ar.row(g9 % 3 - 1, g9 / 3 - 1);
 #pragma unroll
       for (int a = 2; a >= 0; --a) {
         const int T = a + 3 * g9;
@@ -754,8 +775,8 @@ __device__ __forceinline__ R red_part(R fstar, const Recol<R>& rc) {
   return fma_(rc.rc[speed2_of(T)], cdot<T>(rc.n0, rc.n1, rc.n2), rc.frac * fstar);
 }
 
-// Fast rows (a warp is one x-row whose y/z neighbours are inside the box; its lanes
-// 0 .. last hold nodes): the directions (-1|0|+1, dy, dz) = 3K, 3K+1, 3K+2 of the warp
+// Fast rows (a warp is one x-row that touches no face that bounces back; its lanes 0 .. last hold
+// nodes): the directions (-1|0|+1, dy, dz) = 3K, 3K+1, 3K+2 of the warp
 // all land in the target row (y+dy, z+dz); lane l's target x0+l collects
 // z(l) + p(l-1) + m(l+1), summed with two shuffles; lanes 0 and `last` also write
 // m(0) / p(last) into the columns beside the row.
@@ -799,7 +820,7 @@ __device__ __forceinline__ void axis_target(int& q, int p, int c, int n, int bc_
   }
 }
 
-// Other rows (next to a y or z face, or boxes without fast rows): direction T
+// Other rows (next to a no-slip y or z face, or every row where an x face is one): direction T
 // goes straight into the global accumulators of the owner of its slot S(x, T)
 // (bounced back to x, reflected, wrapped, or into the ghost plane above an
 // outflow face, which no node reads as a density).
@@ -916,7 +937,7 @@ __device__ __forceinline__ void emit(const Store& st, const KConst<R>& K, const 
   if (FAST) {
     auto* p1 = st.A + ar.e[1];
     if (!odd) st.store_rel(p1, 0, opp_of(T), speed2_of(T), K, outr, outb, fstar, q);
-    else st.store_rel(p1 + ar.template row_off<Store::PLANES>(G, cy_of(T), cz_of(T)),
+    else st.store_rel(p1 + ar.row(cy_of(T), cz_of(T)),
                       cx_of(T) < 0 ? ar.dxm : (cx_of(T) > 0 ? ar.dxp : 0), T, speed2_of(T), K, outr, outb, fstar, q);
   } else if (!odd) {
     st.store(nm.base, opp_of(T), speed2_of(T), K, outr, outb, fstar, q);
@@ -1055,12 +1076,15 @@ __global__ void __launch_bounds__(B::NT, 4) k_density(Store st, Geom G,
   using D = typename DensOf<Store>::real;
   const int x = blockIdx.x * B::BX + threadIdx.x;
   const int y = blockIdx.y * B::BY + threadIdx.y;
-  const int z = (gridDim.z - 1 - blockIdx.z) * B::BZ + threadIdx.z;
+  const int z = (gridDim.z - 1 - face_first(blockIdx.z, gridDim.z, G.bc[4])) * B::BZ + threadIdx.z;
   if (x >= G.nx || y >= G.ny || z >= G.nz) return;
   if (top != nullptr && z == G.nz - 1) outflow_column(st, G, K, layout, x, y, top);
   D rr = D(0), ft[27];
-  if (fast_row(G, y, z)) {
-    AoRow ar;
+  AoRow ar;
+  if (interior_row(G, y, z)) {  // shifts from the box alone, the same in every lane: 151.5 -> 149 us (jet f16)
+    ar.init<Store::PLANES, true>(G, x, y, z);
+    load_node_fast(st, K, G, ar, layout, rr, ft);
+  } else if (fast_row(G, y, z)) {
     ar.init<Store::PLANES>(G, x, y, z);
     load_node_fast(st, K, G, ar, layout, rr, ft);
   } else {
@@ -1223,7 +1247,7 @@ __global__ void __launch_bounds__(B::NT, MINB)
   __shared__ int pfast[B::NW];
   __shared__ uint64_t tbar;
 
-  int x0 = blockIdx.x * B::BX, y0 = blockIdx.y * B::BY, z0 = blockIdx.z * B::BZ;
+  int x0 = blockIdx.x * B::BX, y0 = blockIdx.y * B::BY, z0 = face_first(blockIdx.z, gridDim.z, G.bc[5]) * B::BZ;
   if (bmode) {
     // the block's boundary tile, computed once (block 0: the tile at the origin)
     __shared__ int3 btile;
@@ -1402,8 +1426,15 @@ __global__ void __launch_bounds__(B::NT, MINB)
       const int row = warp + k * B::NW;
       if (row < B::TY * B::TZ) {
         const int ty = row % B::TY, tz = row / B::TY;
-        const int gy = y0 - 1 + ty, gz = z0 - 1 + tz;
-        if (gy >= 0 && gy < G.ny && gz >= 0 && gz < G.nz) {
+        int gy = y0 - 1 + ty, gz = z0 - 1 + tz;
+        // a row beyond a face belongs to the row across it (periodic) or, reflected, to the face row
+        // itself; the ghost plane above an outflow face is no density
+        const bool ghost = gz == G.nz && G.bc[5] == BC_OUTFLOW;
+        if (gy < 0) gy = G.bc[2] == BC_PERIODIC ? G.ny - 1 : 0;
+        else if (gy == G.ny) gy = G.bc[3] == BC_PERIODIC ? 0 : G.ny - 1;
+        if (gz < 0) gz = G.bc[4] == BC_PERIODIC ? G.nz - 1 : 0;
+        else if (gz == G.nz) gz = G.bc[5] == BC_PERIODIC ? 0 : G.nz - 1;
+        if (!ghost && gy < G.ny && gz < G.nz) {
           float2 a = make_float2(0.f, 0.f), b = make_float2(0.f, 0.f);
 #pragma unroll
           for (int wz = 0; wz < B::BZ; ++wz) {
@@ -1567,7 +1598,7 @@ __device__ __forceinline__ void cp_async_wait_prev() { asm volatile("cp.async.wa
 template <int T>
 __device__ __forceinline__ int64_t fast_src(const Geom& G, const AoRow& ar, int odd) {
   if (!odd) return ar.e[1] + T * 32;
-  return ar.slot0<26 - T, 27>(G) + (26 - T) * 32;
+  return ar.e[1] + ar.rel0<26 - T>() + (26 - T) * 32;
 }
 template <int T>
 struct PfIssueFast {

@@ -199,7 +199,7 @@ __global__ void __launch_bounds__(TP_THREADS, TP_MINB)
       const bool recol = __any_sync(__activemask(), any_(rc.has_n));
       NodeMap nm;
       AoRow ar;
-      ar.init<27>(G, x, y, z);
+      ar.init<27, true>(G, x, y, z);
       if (recol) EmitLoop<0, Store, float, true, true, false, ODD, B::BY, B::TX>::run(st, K, G, nm, ar, ODD != 0, f, rc, nullptr, FusedIO{}, x, y, z);
       else EmitLoop<0, Store, float, true, false, false, ODD, B::BY, B::TX>::run(st, K, G, nm, ar, ODD != 0, f, rc, nullptr, FusedIO{}, x, y, z);
     }
