@@ -240,11 +240,11 @@ __global__ void __launch_bounds__(NTHREADS, 3) k_density_c(CompactStore<BF16> st
   if (!active) return;
   float rho = 0.f, rr = 0.f;
   if (top) {
-    const float* tp = G.ctop + ((int64_t)x + (int64_t)G.nx * y) * 64;
+    const float* tp = G.ctop + top_column(G, x, y);
 #pragma unroll
     for (int t = 0; t < 27; ++t) {
-      rr += tp[t];
-      rho += tp[t] + tp[32 + t];
+      rr += tp[t * 32];
+      rho += tp[t * 32] + tp[(32 + t) * 32];
     }
   } else if (fast) {
     const int lx = threadIdx.x + 1, ly = threadIdx.y + 1, lz = threadIdx.z + 1;
@@ -332,11 +332,11 @@ __device__ __forceinline__ void dens_general(const CompactStore<BF16>& st, const
                                              int x, int y, int z, float2* __restrict__ dens, int* __restrict__ flag) {
   float rho = 0.f, rr = 0.f;
   if (on_top(G, z)) {
-    const float* tp = G.ctop + ((int64_t)x + (int64_t)G.nx * y) * 64;
+    const float* tp = G.ctop + top_column(G, x, y);
 #pragma unroll
     for (int t = 0; t < 27; ++t) {
-      rr += tp[t];
-      rho += tp[t] + tp[32 + t];
+      rr += tp[t * 32];
+      rho += tp[t * 32] + tp[(32 + t) * 32];
     }
   } else {
     NodeMap nm;
@@ -586,9 +586,9 @@ __global__ void __launch_bounds__(NTHREADS, 4)
   const bool fast = fast_row(G, y, z);
   if (active) {
     if (on_top(G, z)) {
-      const float* tp = G.ctop + ((int64_t)x + (int64_t)G.nx * y) * 64;
+      const float* tp = G.ctop + top_column(G, x, y);
 #pragma unroll
-      for (int t = 0; t < 27; ++t) ft[t] = tp[t] + tp[32 + t];
+      for (int t = 0; t < 27; ++t) ft[t] = tp[t * 32] + tp[(32 + t) * 32];
     } else if (fast) {
       AoRow ar;
       ar.init<CPLANES>(G, x, y, z);
@@ -702,40 +702,47 @@ __global__ void __launch_bounds__(NTHREADS, 4)
 
 // convective outflow (Sec. IV.A) on the compact storage: the node below the top plane is read
 // (totals and rebuilt colours), the top plane's per-colour populations live in Geom::ctop only
-template <bool BF16>
-__global__ void __launch_bounds__(256) k_outflow_c(CompactStore<BF16> st, Geom G,
-                                                   const __grid_constant__ KConst<float> K, int layout) {
-  const int64_t Pn = (int64_t)G.nx * G.ny;
-  const int64_t pp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;  // warp-uniform
-  if (pp >= Pn) return;
-  const int lane = threadIdx.x & 31;
-  const bool act = lane < 27;
-  const int t = act ? lane : 0;
-  const int x = (int)(pp % G.nx), y = (int)(pp / G.nx);
-  NodeMap below;
-  below.init(G, x, y, G.nz - 2);
-  float fr = 0.f, fb = 0.f;
-  if (act) {
+// (columns and directions split as in k_outflow)
+template <int W, bool BF16>
+__device__ __forceinline__ void outflow_load_c(const CompactStore<BF16>& st, const KConst<float>& K,
+                                               const NodeMap& below, int layout, float* fr, float* fb) {
+#pragma unroll
+  for (int t = W, k = 0; t < 27; t += OUT_W, ++k) {
     int64_t node, src;
     int dir, sdir;
     slot_of(below, layout, t, node, dir);
     slot_of(below, 1, t, src, sdir);
     const float v = st.load(node, dir, speed2_of(t), K);
-    fr = red_of(v, st.rec[src], opp_of(sdir));
-    fb = v - fr;
+    fr[k] = red_of(v, st.rec[src], opp_of(sdir));
+    fb[k] = v - fr[k];
   }
-  const float v = fr + fb;
-  const float rho = warp_allsum(v);
-  const float mz = warp_allsum(cz_of(t) > 0 && act ? v : cz_of(t) < 0 && act ? -v : 0.f);
-  float F[3];
-  body_force(K, rho, F);
-  const float uz = (mz + 0.5f * F[2]) / rho;
-  const float lam = uz > 0.f ? uz : 0.f;
-  const float inv = 1.f / (1.f + lam);
-  if (act) {
-    float* tr = G.ctop + pp * 64 + t;
-    tr[0] = (tr[0] + lam * fr) * inv;
-    tr[32] = (tr[32] + lam * fb) * inv;
+}
+template <bool BF16>
+__global__ void __launch_bounds__(32 * OUT_W) k_outflow_c(CompactStore<BF16> st, const __grid_constant__ Geom G,
+                                                          const __grid_constant__ KConst<float> K, int layout) {
+  __shared__ OutflowSums<float> sh;
+  int x, y;
+  const bool in = outflow_xy(G, x, y);
+  float* const tr = G.ctop + (in ? top_column(G, x, y) : 0);
+  float fr[OUT_N], fb[OUT_N], hr[OUT_N], hb[OUT_N];
+  if (in) {
+    NodeMap below;
+    below.init(G, x, y, G.nz - 2);
+#define LBMK_OUT_BODY(W)                            \
+  outflow_top<W>(tr, hr, hb);                       \
+  outflow_load_c<W>(st, K, below, layout, fr, fb);  \
+  outflow_moments<W>(sh, fr, fb)
+    LBMK_OUT_WARPS(LBMK_OUT_BODY)
+#undef LBMK_OUT_BODY
+  }
+  __syncthreads();
+  if (in) {
+    float rho, mz, lam, inv;
+    outflow_total(sh, rho, mz);
+    outflow_lambda(K, rho, mz, lam, inv);
+#define LBMK_OUT_BODY(W) outflow_mix<W>(tr, hr, hb, lam, inv, fr, fb)
+    LBMK_OUT_WARPS(LBMK_OUT_BODY)
+#undef LBMK_OUT_BODY
   }
 }
 
@@ -752,13 +759,13 @@ __global__ void k_init_c(CompactStore<BF16> st, Geom G, const __grid_constant__ 
   const double r = rr[n], b = rb[n];
   const int64_t sn = snode(G, x, y, z);
   const bool top = on_top(G, z);
-  float* const tp = G.ctop + ((int64_t)x + (int64_t)G.nx * y) * 64;
+  float* const tp = G.ctop + top_column(G, x, y);
   equilibrium_pairs<DF>(r, b, u ? u[n] : 0.0, u ? u[N + n] : 0.0, u ? u[2 * N + n] : 0.0, K.alpha_r_d,
                         [&](int t, DF fr, DF fb) {
                           st.store(sn, t, speed2_of(t), K, narrow_(add_(fr, fb)));
                           if (top) {
-                            tp[t] = narrow_(fr);
-                            tp[32 + t] = narrow_(fb);
+                            tp[t * 32] = narrow_(fr);
+                            tp[(32 + t) * 32] = narrow_(fb);
                           }
                         });
   dens[n] = make_float2((float)(r + b), (float)((r - b) / (r + b)));
@@ -782,9 +789,9 @@ __global__ void k_macro_c(CompactStore<BF16> st, Geom G, const __grid_constant__
 #pragma unroll
   for (int t = 0; t < 27; ++t) {
     if (top) {
-      const float* tp = G.ctop + ((int64_t)x + (int64_t)G.nx * y) * 64;
-      const DF s = two_sum(tp[t], tp[32 + t]);
-      acc_(sred, tp[t]);
+      const float* tp = G.ctop + top_column(G, x, y);
+      const DF s = two_sum(tp[t * 32], tp[(32 + t) * 32]);
+      acc_(sred, tp[t * 32]);
       acc_(srho, s);
       if (cx_of(t)) acc_(m[0], cx_of(t) > 0 ? s : neg_(s));
       if (cy_of(t)) acc_(m[1], cy_of(t) > 0 ? s : neg_(s));
@@ -826,9 +833,9 @@ __global__ void k_get_pop_c(CompactStore<BF16> st, Geom G, const __grid_constant
   const int x = (int)(n % G.nx), y = (int)((n / G.nx) % G.ny), z = (int)(n / ((int64_t)G.nx * G.ny));
   const int t = paper_to_tensor(pdir);
   if (on_top(G, z)) {
-    const float* tp = G.ctop + ((int64_t)x + (int64_t)G.nx * y) * 64;
-    out_r[n] = tp[t];
-    out_b[n] = tp[32 + t];
+    const float* tp = G.ctop + top_column(G, x, y);
+    out_r[n] = tp[t * 32];
+    out_b[n] = tp[(32 + t) * 32];
     return;
   }
   NodeMap nm;
@@ -858,8 +865,8 @@ __global__ void k_set_pop_c(CompactStore<BF16> st, Geom G, const __grid_constant
   acc_r[n] = (pdir == 0 ? 0.0 : acc_r[n]) + r;
   acc_b[n] = (pdir == 0 ? 0.0 : acc_b[n]) + b;
   if (on_top(G, z)) {
-    G.ctop[((int64_t)x + (int64_t)G.nx * y) * 64 + t] = (float)r;
-    G.ctop[((int64_t)x + (int64_t)G.nx * y) * 64 + 32 + t] = (float)b;
+    G.ctop[top_column(G, x, y) + t * 32] = (float)r;
+    G.ctop[top_column(G, x, y) + (32 + t) * 32] = (float)b;
   }
   NodeMap nm;
   nm.init(G, x, y, z);

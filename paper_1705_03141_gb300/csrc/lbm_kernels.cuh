@@ -175,6 +175,14 @@ __host__ __device__ __forceinline__ int64_t elem_index(int64_t node, int planes,
   return ((node >> 5) * planes + plane) * 32 + (node & 31);
 }
 
+// The outflow plane's per-colour populations: columns (x, y) in blocks of 32, 64 rows a block (27 red
+// from row 0, 27 blue from row 32), so that a warp of columns reads and writes whole lines.
+// Offset of row 0 of a column; row r is 32 r further.
+__host__ __device__ __forceinline__ int64_t top_column(const Geom& g, int x, int y) {
+  const int64_t c = (int64_t)x + (int64_t)g.nx * y;
+  return (c >> 5) * (64 * 32) + (c & 31);
+}
+
 // Per-node streaming map: for each axis and side the node-index offset of the
 // neighbour, whether that side reflects the component (free-slip) and whether
 // it bounces back (no-slip).
@@ -241,7 +249,7 @@ struct NodeMap {
 struct AoRow {
   int64_t e[3];
   int dxm, dxp;        // e[0] - e[1] and e[2] - e[1]
-  int ym, yp, zm, zp;  // row shifts in units of 32 elements (|shift| < 2^31: NodeMap keeps the box below 2^31 nodes)
+  int ym, yp, zm, zp;  // row shifts in units of 32 elements (below 2^31 up to 2.5e9 padded nodes)
   // the node's storage block (x >> 5) + (nxs / 32)(y + ny (z + 1)) fits 32 bits; within a block the
   // x neighbours are one element away, across a block edge one block of PLANES planes minus 31.
   // INTERIOR: the row touches no y or z face
@@ -319,32 +327,6 @@ __device__ __forceinline__ void slot_of(const NodeMap& nm, int layout, int t, in
   }
 }
 
-// slot_of for a direction known only at run time (one lane per direction): the slot map of
-// NodeMap::push written with selects instead of a switch, so the lanes of a warp do not diverge
-__device__ __forceinline__ void slot_of_rt(const NodeMap& nm, int layout, int t, int64_t& node, int& dir) {
-  if (layout == 0) {
-    node = nm.base;
-    dir = t;
-    return;
-  }
-  const int T = 26 - t;  // the slot S(x, opp(t))
-  const int c[3] = {cx_of(T), cy_of(T), cz_of(T)};
-  int off = 0, d = T;
-  bool bounce = false;
-#pragma unroll
-  for (int a = 0; a < 3; ++a) {
-    const unsigned bit = 1u << a;
-    const int sh = a == 0 ? 2 : (a == 1 ? 6 : 18);
-    const bool neg = c[a] < 0, pos = c[a] > 0;
-    off += neg ? nm.off_m[a] : (pos ? nm.off_p[a] : 0);
-    d += (neg && (nm.flip_m & bit)) ? sh : 0;
-    d -= (pos && (nm.flip_p & bit)) ? sh : 0;
-    bounce = bounce || (neg && (nm.bounce_m & bit)) || (pos && (nm.bounce_p & bit));
-  }
-  node = bounce ? nm.base : nm.base + off;
-  dir = bounce ? opp_of(T) : d;
-}
-
 // ---------------------------------------------------------------------------
 // storage policies.  `cls` is the speed class |c|^2 of the direction; it is
 // unchanged by reflection and bounce-back, so the hot kernels pass it as a
@@ -404,9 +386,13 @@ struct PlainStore {  // FP64 or FP32: f^r and f^b planes [2][27][Ns]
   }
   // the two colours as stored (I/O kernels)
   template <typename R>
-  __device__ __forceinline__ void load_rb(int64_t node, int dir, int, const KConst<R>&, R& fr, R& fb) const {
-    fr = (R)A[elem_index(node, PLANES, dir)];
-    fb = (R)A[elem_index(node, PLANES, 27 + dir)];
+  __device__ __forceinline__ void load_rb(int64_t node, int dir, int, const KConst<R>& K, R& fr, R& fb) const {
+    load_rb_at(elem_index(node, PLANES, 0), dir, 0, K, fr, fb);
+  }
+  template <typename R>
+  __device__ __forceinline__ void load_rb_at(int64_t e0, int dir, int, const KConst<R>&, R& fr, R& fb) const {
+    fr = (R)A[e0 + dir * 32];
+    fb = (R)A[e0 + (27 + dir) * 32];
   }
   // outr, outb: the two colours; fstar = outr + outb and q = outr / fstar are for packed storage
   template <typename R>
@@ -529,8 +515,12 @@ struct PackedStore {
   }
   template <typename R>
   __device__ __forceinline__ void load_rb(int64_t node, int dir, int cls, const KConst<R>& K, R& fr, R& fb) const {
+    load_rb_at(elem_index(node, PLANES, 0), dir, cls, K, fr, fb);
+  }
+  template <typename R>
+  __device__ __forceinline__ void load_rb_at(int64_t e0, int dir, int cls, const KConst<R>& K, R& fr, R& fb) const {
     R ft;
-    load(node, dir, cls, K, fr, ft);
+    load_at(e0, dir, cls, K, fr, ft);
     fb = ft - fr;
   }
   template <typename R>
@@ -986,8 +976,7 @@ __device__ __forceinline__ void store_pair(const Store& st, const KConst<R>& K, 
   st.store(node, dir, speed2_of(dir), K, fr, fb, s, q);
 }
 
-// the sum a warp_allsum over lanes 0..31 gives, with v[l] the value of lane l (the same
-// additions in the same order: at each stage lane l adds the value of lane l ^ o); v is consumed
+// the sum of v[0..31] as a binary tree of the pairs (l, l + 16), (l, l + 8), ...; v is consumed
 template <typename R>
 __device__ __forceinline__ R xor_tree_sum(R v[32]) {
 #pragma unroll
@@ -998,47 +987,96 @@ __device__ __forceinline__ R xor_tree_sum(R v[32]) {
   return v[0];
 }
 
-// The convective outflow of the step before (Sec. IV.A) for the column (x, y), by one thread:
-// the same arithmetic, in the same order, as k_outflow (which gives it to 27 lanes); `layout`
-// is the layout of the state the outflow completes.
-template <class Store, typename R>
-__device__ __forceinline__ void outflow_column(const Store& st, const Geom& G, const KConst<R>& K, int layout, int x,
-                                               int y, R* __restrict__ top) {
-  NodeMap below, here;
-  below.init(G, x, y, G.nz - 2);
-  here.init(G, x, y, G.nz - 1);
-  R fr[27], fb[27], a[32], m[32];
-#pragma unroll
-  for (int t = 0; t < 27; ++t) {
-    int64_t node;
-    int dir;
-    slot_of(below, layout, t, node, dir);
-    st.load_rb(node, dir, speed2_of(t), K, fr[t], fb[t]);
-    const R v = fr[t] + fb[t];
-    a[t] = v;
-    m[t] = cz_of(t) > 0 ? v : cz_of(t) < 0 ? -v : R(0);
-  }
-#pragma unroll
-  for (int t = 27; t < 32; ++t) a[t] = m[t] = R(0);
-  const R rho = xor_tree_sum(a);
-  const R mz = xor_tree_sum(m);
+// lambda = max(0, u_z) and 1 / (1 + lambda) from the density and z momentum of the node below the
+// outflow plane
+template <typename R>
+__device__ __forceinline__ void outflow_lambda(const KConst<R>& K, R rho, R mz, R& lam, R& inv) {
   R F[3];
   body_force(K, rho, F);
   const R uz = (mz + R(0.5) * F[2]) / rho;
-  const R lam = uz > R(0) ? uz : R(0);
-  const R inv = R(1) / (R(1) + lam);
-  R* tr = top + ((int64_t)x + (int64_t)G.nx * y) * 64;
+  lam = uz > R(0) ? uz : R(0);
+  inv = R(1) / (R(1) + lam);
+}
+
+// The directions t = W, W + STEP, ... of a column (x, y) of the outflow plane: the populations of the
+// node below, and the new ones of the plane's node into its slots (layout: of the state that the
+// outflow completes).
+template <int W, int STEP, class Store, typename R>
+__device__ __forceinline__ void outflow_load(const Store& st, const Geom& G, const KConst<R>& K, int layout, int x,
+                                             int y, R* fr, R* fb) {
+  if (fast_row(G, y, G.nz - 2)) {
+    AoRow ar;
+    ar.init<Store::PLANES>(G, x, y, G.nz - 2);
+#pragma unroll
+    for (int t = W, k = 0; t < 27; t += STEP, ++k) {
+      const int T = 26 - t;
+      if (!layout) st.load_rb_at(ar.e[1], t, speed2_of(t), K, fr[k], fb[k]);
+      else st.load_rb_at(ar.e[cx_of(T) + 1] + ar.row(cy_of(T), cz_of(T)), T, speed2_of(t), K, fr[k], fb[k]);
+    }
+  } else {
+    NodeMap below;
+    below.init(G, x, y, G.nz - 2);
+#pragma unroll
+    for (int t = W, k = 0; t < 27; t += STEP, ++k) {
+      int64_t node;
+      int dir;
+      slot_of(below, layout, t, node, dir);
+      st.load_rb(node, dir, speed2_of(t), K, fr[k], fb[k]);
+    }
+  }
+}
+template <int W, int STEP, class Store, typename R>
+__device__ __forceinline__ void outflow_store(const Store& st, const Geom& G, const KConst<R>& K, int layout, int x,
+                                              int y, const R* fr, const R* fb) {
+  if (fast_row(G, y, G.nz - 1)) {
+    AoRow ar;
+    ar.init<Store::PLANES>(G, x, y, G.nz - 1);
+#pragma unroll
+    for (int t = W, k = 0; t < 27; t += STEP, ++k) {
+      const int T = 26 - t;
+      const R s = fr[k] + fb[k];
+      const R q = s > R(0) ? fr[k] / s : R(0.5);
+      if (!layout) st.store_at(ar.e[1], t, speed2_of(t), K, fr[k], fb[k], s, q);
+      else st.store_at(ar.e[cx_of(T) + 1] + ar.row(cy_of(T), cz_of(T)), T, speed2_of(t), K, fr[k], fb[k], s, q);
+    }
+  } else {
+    NodeMap here;
+    here.init(G, x, y, G.nz - 1);
+#pragma unroll
+    for (int t = W, k = 0; t < 27; t += STEP, ++k) {
+      int64_t node;
+      int dir;
+      slot_of(here, layout, t, node, dir);
+      store_pair(st, K, node, dir, fr[k], fb[k]);
+    }
+  }
+}
+
+// The convective outflow of the step before (Sec. IV.A) for the column (x, y), by one thread: the same
+// arithmetic, in the same order, as k_outflow (which gives it to four)
+template <class Store, typename R>
+__device__ __forceinline__ void outflow_column(const Store& st, const Geom& G, const KConst<R>& K, int layout, int x,
+                                               int y, R* __restrict__ top) {
+  R fr[27], fb[27], a[32], m[32];
+  outflow_load<0, 1>(st, G, K, layout, x, y, fr, fb);
+#pragma unroll
+  for (int t = 0; t < 32; ++t) {
+    const R v = t < 27 ? fr[t % 27] + fb[t % 27] : R(0);
+    a[t] = v;
+    m[t] = t < 27 && cz_of(t) > 0 ? v : t < 27 && cz_of(t) < 0 ? -v : R(0);
+  }
+  R lam, inv;
+  const R rho = xor_tree_sum(a), mz = xor_tree_sum(m);
+  outflow_lambda(K, rho, mz, lam, inv);
+  R* const tr = top + top_column(G, x, y);
 #pragma unroll
   for (int t = 0; t < 27; ++t) {
-    const R nr = (tr[t] + lam * fr[t]) * inv;
-    const R nb = (tr[32 + t] + lam * fb[t]) * inv;
-    tr[t] = nr;
-    tr[32 + t] = nb;
-    int64_t node;
-    int dir;
-    slot_of(here, layout, t, node, dir);
-    store_pair(st, K, node, dir, nr, nb);
+    fr[t] = (tr[t * 32] + lam * fr[t]) * inv;
+    fb[t] = (tr[(32 + t) * 32] + lam * fb[t]) * inv;
+    tr[t * 32] = fr[t];
+    tr[(32 + t) * 32] = fb[t];
   }
+  outflow_store<0, 1>(st, G, K, layout, x, y, fr, fb);
 }
 
 // (rho, phi) of a node from its red density and totals; inlet: a Dirichlet inlet node
@@ -1891,72 +1929,135 @@ __global__ void __launch_bounds__(PTHREADS, MINB)
 }
 
 
-// sum over the 32 lanes of a warp, the same value in every lane (butterfly: lanes i and i^o
-// hold the same partial sum at every stage, as addition commutes exactly)
-template <typename R>
-__device__ __forceinline__ R warp_allsum(R v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
+// Convective outflow on the z = nz-1 plane (Sec. IV.A), after the step that produced time t+1;
+// `layout` is the layout of time t+1: f(N, t+1) = (f(N, t) + lambda f(N-1, t+1)) / (1 + lambda) for
+// every direction and colour, lambda = max(0, u_z(N-1, t+1)); `top` holds f(N, t) and is updated.
+// The plane holds only nx ny nodes, so the kernel is a few trips to memory, one after another, and
+// what counts is that a warp's accesses are whole lines and that no thread has much to do: a block is 32
+// columns along x by 4 warps, and warp w takes the directions t = w, w + 4, ... of its columns.
+// The sums over the directions pair t with t + 16, t + 8 and t + 4 first, which is inside a
+// warp's share, and t + 2 and t + 1 through shared memory (the order of xor_tree_sum).
+// Against one warp per column with a direction in each lane, which touched a sector for every 4 bytes,
+// us a step: 128x128x512 compact 567 -> 545, FP32 777 -> 773, 200x200x600 FP32 2438 -> 2425;
+// in pass 1 (outflow_column) 32x32x64 f16 27.2 -> 23.9, 66x20x40 FP32 22.9 -> 18.4.
+constexpr int OUT_W = 4, OUT_N = 7;  // warps of a block; directions of a thread
+inline dim3 outflow_block() { return dim3(32, OUT_W); }
+inline unsigned outflow_grid(const Geom& G) { return (unsigned)((G.nx + 31) / 32) * G.ny; }
+__device__ __forceinline__ bool outflow_xy(const Geom& G, int& x, int& y) {
+  const int ntx = (G.nx + 31) / 32;
+  y = blockIdx.x / ntx;
+  x = (blockIdx.x - y * ntx) * 32 + threadIdx.x;
+  return x < G.nx;
 }
-
-// convective outflow on the z = nz-1 plane (Sec. IV.A), after the step that
-// produced time t+1; `layout` is the layout of time t+1.  One warp per column
-// (x, y), lane t < 27 for direction t (the plane holds only nx ny nodes: a
-// thread per node would leave most of the SMs idle and run each column's 27
-// directions one after another); the slot map uses selects, so the lanes do not
-// diverge.  The lanes reduce rho and the z momentum of the node below with
-// shuffles, then each sets f(N, t+1) = (f(N, t) + lambda f(N-1, t+1)) /
-// (1 + lambda) for its direction and both colours, lambda = max(0, u_z(N-1, t+1));
-// `top` holds f(N, t) per column (32 red then 32 blue slots), and is updated.
-template <class Store>
-__global__ void __launch_bounds__(256) k_outflow(Store st, Geom G,
-                                                 const __grid_constant__ KConst<typename DensOf<Store>::real> K,
-                                                 int layout, typename DensOf<Store>::real* __restrict__ top,
-                                                 unsigned long long* __restrict__ fix) {
-  using R = typename DensOf<Store>::real;
-  const int64_t Pn = (int64_t)G.nx * G.ny;
-  const int64_t pp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;  // warp-uniform
-  if (pp >= Pn) return;
-  const int lane = threadIdx.x & 31;
-  const bool act = lane < 27;
-  const int t = act ? lane : 0;
-  const int x = (int)(pp % G.nx), y = (int)(pp / G.nx);
-  NodeMap below, here;
-  below.init(G, x, y, G.nz - 2);
-  here.init(G, x, y, G.nz - 1);
-  R fr = R(0), fb = R(0);
-  if (act) {
-    int64_t node;
-    int dir;
-    slot_of_rt(below, layout, t, node, dir);
-    st.load_rb(node, dir, speed2_of(t), K, fr, fb);
+template <typename R>
+struct OutflowSums {
+  R a[OUT_W][32], m[OUT_W][32];
+};
+// the sums over all directions of a and of m, each given for the directions of the thread
+template <int W, typename R>
+__device__ __forceinline__ void outflow_part(OutflowSums<R>& sh, const R* a, const R* m) {
+  R u[8], v[8];
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    const bool in = W + 4 * k < 27;
+    u[k] = in ? a[k % OUT_N] : R(0);
+    v[k] = in ? m[k % OUT_N] : R(0);
   }
-  const R v = fr + fb;
-  const R rho = warp_allsum(v);
-  const R mz = warp_allsum(cz_of(t) > 0 && act ? v : cz_of(t) < 0 && act ? -v : R(0));
-  R F[3];
-  body_force(K, rho, F);
-  const R uz = (mz + R(0.5) * F[2]) / rho;
-  const R lam = uz > R(0) ? uz : R(0);
-  const R inv = R(1) / (R(1) + lam);
-  R nr = R(0), nb = R(0);
-  if (act) {
-    R* tr = top + pp * 64 + t;  // per column: 32 red then 32 blue slots, one line per warp
-    R* tb = tr + 32;
-    nr = (*tr + lam * fr) * inv;
-    nb = (*tb + lam * fb) * inv;
-    *tr = nr;
-    *tb = nb;
-    int64_t node;
-    int dir;
-    slot_of_rt(here, layout, t, node, dir);
-    store_pair(st, K, node, dir, nr, nb);
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1) {
+#pragma unroll
+    for (int k = 0; k < o; ++k) {
+      u[k] += u[k + o];
+      v[k] += v[k + o];
+    }
+  }
+  sh.a[W][threadIdx.x] = u[0];
+  sh.m[W][threadIdx.x] = v[0];
+}
+template <typename R>
+__device__ __forceinline__ void outflow_total(const OutflowSums<R>& sh, R& a, R& m) {
+  const int l = threadIdx.x;
+  a = (sh.a[0][l] + sh.a[2][l]) + (sh.a[1][l] + sh.a[3][l]);
+  m = (sh.m[0][l] + sh.m[2][l]) + (sh.m[1][l] + sh.m[3][l]);
+}
+// the density and z momentum of the node below from the thread's directions
+template <int W, typename R>
+__device__ __forceinline__ void outflow_moments(OutflowSums<R>& sh, const R* fr, const R* fb) {
+  R a[OUT_N], m[OUT_N];
+#pragma unroll
+  for (int t = W, k = 0; t < 27; t += OUT_W, ++k) {
+    a[k] = fr[k] + fb[k];
+    m[k] = cz_of(t) > 0 ? a[k] : cz_of(t) < 0 ? -a[k] : R(0);
+  }
+  outflow_part<W>(sh, a, m);
+}
+template <int W, typename R>
+__device__ __forceinline__ void outflow_top(const R* tr, R* hr, R* hb) {
+#pragma unroll
+  for (int t = W, k = 0; t < 27; t += OUT_W, ++k) {
+    hr[k] = tr[t * 32];
+    hb[k] = tr[(32 + t) * 32];
+  }
+}
+// the new populations of the plane's node, into `top`
+template <int W, typename R>
+__device__ __forceinline__ void outflow_mix(R* tr, const R* hr, const R* hb, R lam, R inv, R* fr, R* fb) {
+#pragma unroll
+  for (int t = W, k = 0; t < 27; t += OUT_W, ++k) {
+    tr[t * 32] = fr[k] = (hr[k] + lam * fr[k]) * inv;
+    tr[(32 + t) * 32] = fb[k] = (hb[k] + lam * fb[k]) * inv;
+  }
+}
+#define LBMK_OUT_WARPS(BODY) \
+  switch (threadIdx.y) {     \
+    case 0: BODY(0); break;  \
+    case 1: BODY(1); break;  \
+    case 2: BODY(2); break;  \
+    default: BODY(3); break; \
+  }
+
+template <class Store>
+__global__ void __launch_bounds__(32 * OUT_W)
+    k_outflow(Store st, const __grid_constant__ Geom G,
+              const __grid_constant__ KConst<typename DensOf<Store>::real> K, int layout,
+              typename DensOf<Store>::real* __restrict__ top, unsigned long long* __restrict__ fix) {
+  using R = typename DensOf<Store>::real;
+  __shared__ OutflowSums<R> sh, shf;
+  int x, y;
+  const bool in = outflow_xy(G, x, y);
+  R* const tr = top + (in ? top_column(G, x, y) : 0);
+  R fr[OUT_N], fb[OUT_N], hr[OUT_N], hb[OUT_N];
+  if (in) {
+#define LBMK_OUT_BODY(W)                                       \
+  outflow_top<W>(tr, hr, hb);                                  \
+  outflow_load<W, OUT_W>(st, G, K, layout, x, y, fr, fb);      \
+  outflow_moments<W>(sh, fr, fb)
+    LBMK_OUT_WARPS(LBMK_OUT_BODY)
+#undef LBMK_OUT_BODY
+  }
+  __syncthreads();
+  if (in) {
+    R rho, mz, lam, inv;
+    outflow_total(sh, rho, mz);
+    outflow_lambda(K, rho, mz, lam, inv);
+#define LBMK_OUT_BODY(W)                                       \
+  outflow_mix<W>(tr, hr, hb, lam, inv, fr, fb);                \
+  outflow_store<W, OUT_W>(st, G, K, layout, x, y, fr, fb);     \
+  if (fix) {                                                   \
+    _Pragma("unroll") for (int k = 0; k < OUT_N; ++k) fb[k] = fr[k] + fb[k]; \
+    outflow_part<W>(shf, fb, fr);                              \
+  }
+    LBMK_OUT_WARPS(LBMK_OUT_BODY)
+#undef LBMK_OUT_BODY
   }
   // fused density pass: the plane's new populations replace what the collide-stream kernel accumulated
   if (fix) {
-    const R sr = warp_allsum(nr), sa = warp_allsum(nr + nb);
-    if (lane == 0) fix[dnode(G, x, y, G.nz - 1)] = pack_fix((float)sa, (float)sr, (float)K.fix_scale);
+    __syncthreads();
+    if (in && threadIdx.y == 0) {
+      R rho, rr;
+      outflow_total(shf, rho, rr);
+      fix[dnode(G, x, y, G.nz - 1)] = pack_fix((float)rho, (float)rr, (float)K.fix_scale);
+    }
   }
 }
 
@@ -2078,8 +2179,9 @@ __global__ void k_top_from_state(Store st, Geom G, const __grid_constant__ KCons
     slot_of(nm, layout, t, node, dir);
     R fr, fb;
     st.load_rb(node, dir, speed2_of(t), K, fr, fb);
-    top[pp * 64 + t] = fr;  // per column: 32 red then 32 blue slots (27 used)
-    top[pp * 64 + 32 + t] = fb;
+    R* const tr = top + top_column(G, (int)(pp % G.nx), (int)(pp / G.nx));
+    tr[t * 32] = fr;
+    tr[(32 + t) * 32] = fb;
   }
 }
 

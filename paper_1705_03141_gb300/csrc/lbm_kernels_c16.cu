@@ -78,8 +78,8 @@ struct LaunchCompact {
     return cudaGetLastError();
   }
   static cudaError_t outflow(void* pop, const Geom& G, const Phys& P, int layout, void*, void*, cudaStream_t s) {
-    const int64_t warps = (int64_t)G.nx * G.ny;
-    k_outflow_c<B><<<blocks1(warps * 32, 256), 256, 0, s>>>(make(pop, G), G, kc(P), layout);
+    k_outflow_c<B><<<outflow_grid(G), outflow_block(), 0, s>>>(
+        make(pop, G), G, kc(P), layout);
     return cudaGetLastError();
   }
   static cudaError_t get_pop(void* pop, const Geom& G, const Phys& P, int layout, int pdir, double* out_r,
