@@ -144,8 +144,8 @@ typedef struct {
                             allocates (cudaMalloc) and frees it itself. */
   size_t workspace_bytes;
   int variant;           /* collide-stream kernel: 0 = library's choice (3 for F32
-                            storage with nx a multiple of 32 or at least 2^20
-                            nodes, 5 for F16/BF16 storage, 1 otherwise: the
+                            storage with nx a multiple of 32 or, by size, where
+                            it is faster, 5 for F16/BF16 storage, 1 otherwise: the
                             measured faster ones; slab handles 1 for F32),
                             1 = one node per thread, 2 = two x-adjacent nodes per
                             thread with packed FP32x2 arithmetic (needs F32/F16/BF16

@@ -105,6 +105,19 @@ bool pipelined_ok(int nx, int ny, int nz, const lbm_params* p) {
          p->bc[1] != LBM_BC_NOSLIP && nx % 32 != 1 && ny > 2 * lbmk::BY && nz > 2 * lbmk::BZ;
 }
 
+// where FP32 storage runs the fused density pass: its collide-stream kernel is bound by memory, so
+// that dropping pass 1 pays, always where rows fill whole 32-node blocks.  Ragged rows leave lanes of the
+// (longer) fused kernel idle, and pass 1 finds much of a small box in L2, so there it depends on the
+// size; us a step, fused / two passes, no outflow face: 41^3 15.1 / 14.5, 60^3 26.2 / 24.9, 70^3 47.7 /
+// 47.0, 75^3 55.6 / 57.6, 80^3 59.2 / 63.0, 85^3 70.4 / 77.0, 97^3 121 / 128, 120^3 170 / 191.  An outflow face adds
+// the outflow kernel to each fused step, while the two passes fold it into pass 1, where it is the
+// tail on small boxes: 66x20x40 14.8 / 18.4, 50x50x100 36.4 / 38.7, 90x90x120 121 / 111,
+// 110x100x100 143 / 134, 120^3 180 / 187, 100x100x200 265 / 277, 200x200x500 2048 / 2277.
+bool fused_pays(int nx, int64_t N, bool outflow) {
+  if (nx % 32 == 0) return true;
+  return outflow ? N < (1 << 18) || N >= (3 << 19) : N >= (3 << 17);
+}
+
 const char* validate(int nx, int ny, int nz, const lbm_params* p) {
   if (!p) return "params is NULL";
   if (nx < 3 || ny < 3 || nz < 3) return "each box dimension must be >= 3";
@@ -380,23 +393,19 @@ lbm_status lbm_create(int nx, int ny, int nz, const lbm_params* p, lbm** out) {
   int64_t Ns = 0;
   h->L = plan(nx, ny, nz, p, h->ks, &Ns, &h->diag_blocks);
   h->stream = static_cast<cudaStream_t>(p->cuda_stream);
-  // default, as measured on GB300: FP32 storage runs the fused density pass (its collide-stream
-  // kernel is bandwidth-bound, so dropping the separate density pass pays) when rows fill whole
-  // 32-node blocks, and with ragged rows from a million nodes on, where the populations no longer
-  // fit in L2 (us a step, fused against two passes: 200x200x500 2048 / 2277, 100x90x300 361 / 378,
-  // 80x80x320 234 / 242, but 85^3 79.7 / 77.3, 41^3 19.2 / 15.5); the packed storages run the
-  // two-pass scheme with the TMA-pipelined collide-stream
-  // kernel on the interior tiles (variant 5: 0.384 against 0.394 ms for the one-node kernel on
-  // the 128x128x512 jet; it runs variant 1 where it does not apply) and FP64 one node per
-  // thread (the fused accumulation costs the packed kernels more than the density pass); the two-node
-  // kernel's register footprint leaves 8 warps per SM and measured slower everywhere
+  // default, as measured on GB300: FP32 storage runs the fused density pass where fused_pays; the
+  // packed storages run the two-pass scheme with the TMA-pipelined collide-stream kernel on
+  // the interior tiles (variant 5; variant 1 where it does not apply: 346 against 361 us for the pass on the
+  // 128x128x512 jet; the fused accumulation costs the packed kernels more than the density pass), FP64
+  // one node per thread; the two-node kernel's register footprint leaves 8 warps per SM and
+  // measured slower everywhere
   h->halo = p->bc[4] == LBM_BC_HALO || p->bc[5] == LBM_BC_HALO;
   h->half = 0;
   h->recs_valid = false;
   h->dens_ready = false;
   const bool packed = p->storage == LBM_STORE_F16 || p->storage == LBM_STORE_BF16;
   h->variant = p->variant != 0 ? p->variant
-                               : (p->storage == LBM_STORE_F32 && (nx % 32 == 0 || h->N >= (1 << 20)) && !h->halo
+                               : (p->storage == LBM_STORE_F32 && !h->halo && fused_pays(nx, h->N, p->bc[5] == LBM_BC_OUTFLOW)
                                       ? 3
                                       : (packed ? 5 : 1));
   h->fix_ready = false;

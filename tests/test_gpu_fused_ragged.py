@@ -54,7 +54,9 @@ def test_fused_ragged_rows(cuda, shape, faces):
 
 
 def test_library_choice_by_size(cuda):
-    for shape, variant in (((64, 20, 40), 3), ((66, 20, 40), 1), ((126, 104, 81), 3)):
-        lat = pkg.Lattice(shape, _work(shape, "periodic")["params"], storage="f32")
+    for shape, faces, variant in (((64, 20, 40), "periodic", 3), ((66, 20, 40), "periodic", 1),
+                                  ((126, 104, 41), "periodic", 3), ((66, 20, 40), "jet", 3),
+                                  ((126, 104, 41), "jet", 1), ((126, 104, 121), "jet", 3)):
+        lat = pkg.Lattice(shape, _work(shape, faces)["params"], storage="f32")
         assert lat.variant == variant
         lat.close()
