@@ -293,7 +293,7 @@ __global__ void __launch_bounds__(NTHREADS, 3) k_density_c(CompactStore<BF16> st
 // AoRow), and the record of the face node with m_x reversed (per-lane offsets and signs).
 // Coordinates outside the box read zeros.  Rows that are not fast rows (next to a y or z face, or
 // the outflow plane) are left out of the tiles, so no tile waits on global-memory latency: before
-// their first tile, all consumer warps of the grid share those rows on the general per-node path
+// their first tile, all consumer warps of the grid share those rows from global memory (dens_general)
 // from global memory, while the producers fill the first stages.  Periodic x faces keep the
 // one-block-per-tile kernel for the whole box.
 struct DcMaps {
@@ -800,6 +800,7 @@ __global__ void k_init_c(CompactStore<BF16> st, Geom G, const __grid_constant__ 
 
 // rho_r, rho_b, u (Eq. Momentum) into FP64 device buffers (any may be null); rho_r from the
 // (rho, phi) field of pass 1 for the current state
+// (128x128x512: 1360 us with every node on the general map and the outflow plane's test in the loop, 600 now)
 template <bool BF16>
 __global__ void k_macro_c(CompactStore<BF16> st, Geom G, const __grid_constant__ KConst<float> K, int layout,
                           const float2* __restrict__ dens, double* __restrict__ rr, double* __restrict__ rb,
@@ -809,27 +810,38 @@ __global__ void k_macro_c(CompactStore<BF16> st, Geom G, const __grid_constant__
   if (n >= N) return;
   const int x = (int)(n % G.nx), y = (int)((n / G.nx) % G.ny), z = (int)(n / ((int64_t)G.nx * G.ny));
   const bool top = on_top(G, z);
-  NodeMap nm;
-  nm.init(G, x, y, z);
   DF srho = {0.f, 0.f}, sred = {0.f, 0.f}, m[3] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
   float f[27];
+  if (top) {
+    const float* tp = G.ctop + top_column(G, x, y);
 #pragma unroll
-  for (int t = 0; t < 27; ++t) {
-    if (top) {
-      const float* tp = G.ctop + top_column(G, x, y);
+    for (int t = 0; t < 27; ++t) {
       const DF s = two_sum(tp[t * 32], tp[(32 + t) * 32]);
       acc_(sred, tp[t * 32]);
       acc_(srho, s);
       if (cx_of(t)) acc_(m[0], cx_of(t) > 0 ? s : neg_(s));
       if (cy_of(t)) acc_(m[1], cy_of(t) > 0 ? s : neg_(s));
       if (cz_of(t)) acc_(m[2], cz_of(t) > 0 ? s : neg_(s));
-    } else {
-      int64_t node;
-      int dir;
-      slot_of(nm, layout, t, node, dir);
-      f[t] = st.load(node, dir, speed2_of(t), K);
-      acc_(srho, f[t]);
     }
+  } else {
+    if (fast_row(G, y, z)) {
+      AoRow ar;
+      ar.init<CPLANES>(G, x, y, z);
+      if (!layout) fast_totals<0>(st, G, K, ar, f);
+      else fast_totals<1>(st, G, K, ar, f);
+    } else {
+      NodeMap nm;
+      nm.init(G, x, y, z);
+#pragma unroll
+      for (int t = 0; t < 27; ++t) {
+        int64_t node;
+        int dir;
+        slot_of(nm, layout, t, node, dir);
+        f[t] = st.load(node, dir, speed2_of(t), K);
+      }
+    }
+#pragma unroll
+    for (int t = 0; t < 27; ++t) acc_(srho, f[t]);
   }
   if (!top && u) {
 #pragma unroll

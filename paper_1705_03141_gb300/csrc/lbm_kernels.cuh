@@ -2197,7 +2197,8 @@ __device__ __forceinline__ void write_velocity(const KConst<R>& K, T rho, const 
     u[a * N + n] = to_f64(div_(mad_(k, wide_<T>(0.5 * (double)K.g[a]), j[a]), rho));
 }
 
-// rho_r, rho_b, u (Eq. Momentum) into FP64 device buffers (any may be null)
+// rho_r, rho_b, u (Eq. Momentum) into FP64 device buffers (any may be null); on the 128x128x512 jet f16
+// 692 -> 567 us, FP32 632 -> 567 against the general map on every node
 template <class Store>
 __global__ void k_macro(Store st, Geom G, const __grid_constant__ KConst<typename DensOf<Store>::real> K, int layout,
                         double* __restrict__ rr, double* __restrict__ rb, double* __restrict__ u) {
@@ -2206,15 +2207,30 @@ __global__ void k_macro(Store st, Geom G, const __grid_constant__ KConst<typenam
   const int64_t n = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (n >= N) return;
   const int x = (int)(n % G.nx), y = (int)((n / G.nx) % G.ny), z = (int)(n / ((int64_t)G.nx * G.ny));
-  NodeMap nm;
-  nm.init(G, x, y, z);
   R fr[27], fb[27];
+  if (fast_row(G, y, z)) {
+    AoRow ar;
+    ar.init<Store::PLANES>(G, x, y, z);
+    if (!layout) {
 #pragma unroll
-  for (int t = 0; t < 27; ++t) {
-    int64_t node;
-    int dir;
-    slot_of(nm, layout, t, node, dir);
-    st.load_rb(node, dir, speed2_of(t), K, fr[t], fb[t]);
+      for (int t = 0; t < 27; ++t) st.load_rb_at(ar.e[1], t, speed2_of(t), K, fr[t], fb[t]);
+    } else {
+#pragma unroll
+      for (int t = 0; t < 27; ++t) {
+        const int T = 26 - t;
+        st.load_rb_at(ar.e[cx_of(T) + 1] + ar.row(cy_of(T), cz_of(T)), T, speed2_of(t), K, fr[t], fb[t]);
+      }
+    }
+  } else {
+    NodeMap nm;
+    nm.init(G, x, y, z);
+#pragma unroll
+    for (int t = 0; t < 27; ++t) {
+      int64_t node;
+      int dir;
+      slot_of(nm, layout, t, node, dir);
+      st.load_rb(node, dir, speed2_of(t), K, fr[t], fb[t]);
+    }
   }
   using T = typename WideOf<R>::type;
   T sr = wide_<T>(0.0), sb = wide_<T>(0.0);
