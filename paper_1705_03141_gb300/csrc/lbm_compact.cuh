@@ -293,8 +293,8 @@ __global__ void __launch_bounds__(NTHREADS, 3) k_density_c(CompactStore<BF16> st
 // AoRow), and the record of the face node with m_x reversed (per-lane offsets and signs).
 // Coordinates outside the box read zeros.  Rows that are not fast rows (next to a y or z face, or
 // the outflow plane) are left out of the tiles, so no tile waits on global-memory latency: before
-// their first tile, all consumer warps of the grid share those rows from global memory (dens_general)
-// from global memory, while the producers fill the first stages.  Periodic x faces keep the
+// their first tile, all consumer warps of the grid share those rows, read from global memory
+// (dens_general), while the producers fill the first stages.  Periodic x faces keep the
 // one-block-per-tile kernel for the whole box.
 struct DcMaps {
   CUtensorMap rest;  // totals as a 5-d tensor (word, plane, block, y, z + 1): box 32 x 1 x 1 x BY x BZ
