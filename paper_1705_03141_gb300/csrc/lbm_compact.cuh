@@ -688,7 +688,7 @@ __global__ void __launch_bounds__(NTHREADS, 4)
   } else {
     const float2 c = tile[lx + TX * (ly + TY * lz)];
     const float rho_r = 0.5f * c.x * (1.f + c.y);
-    const Recol<float> rc = collide<true>(K, rho_r, ft, gphi, grho, f);
+    const Recol<float> rc = collide<false>(K, rho_r, ft, gphi, grho, f);
     record = make_float4(rc.frac, rc.cr * rc.n0, rc.cr * rc.n1, rc.cr * rc.n2);
   }
   st.rec[snode(G, x, y, z)] = record;

@@ -1586,7 +1586,7 @@ __global__ void __launch_bounds__(LIN_THREADS)
     rc.rho = R(1);
     rc.has_n = false;
   } else {
-    rc = collide<true>(K, rho_r, ft, gphi, grho, f);
+    rc = collide<false>(K, rho_r, ft, gphi, grho, f);
   }
   if (__any_sync(mask, any_(rc.has_n))) emit_pairs<0, true>(st, K, nm, odd != 0, f, rc);
   else emit_pairs<0, false>(st, K, nm, odd != 0, f, rc);

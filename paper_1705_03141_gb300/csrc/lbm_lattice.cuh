@@ -335,10 +335,16 @@ inline RelaxConst<R> make_relax(const double rate[27]) {
 //   <a> = F_a,  <a^2> = pi_a - |m|,  <b^2c^2> = (sum pi - |m| - pi_a)/3,  <222> = (sum pi - |m|)/9,
 //   <ab> = u_a F_b + u_b F_a + m_a n_b = 3 <abc^2>,  <ab^2> = <ac^2> = 3 <ab^2c^2> = F_a/3.
 // FOLD: each moment as a scaled moment plus a scaled equilibrium (about 170 operations); otherwise as
-// itself plus its change (about 190), which rounds it once at its own size.  FP32 storage takes the
-// second: folded, its fields came out 3 to 13 % further from FP64, against 15 % nearer than with
-// the moment-by-moment form below.  The 16-bit storages, whose own rounding is 2^12 times larger, and FP64
-// (7.5e-14 either way) take the first: 3 % of a step.
+// itself plus its change (about 190), which rounds it once at its own size.  Error against FP64 relative to
+// relaxing the 23 moments one by one (below), folded / rounded once, geometric means over droplets, jets and
+// Rayleigh-Taylor boxes of several seeds:
+//   FP64 storage, u 1.00 / 0.90, red density 0.98 / 0.97, blue 1.04 / 0.98;
+//   FP32 storage, u 1.03 / 0.85, red density 1.05 / 0.98, blue 1.13 / 0.98;
+//   compact half, red density 1.007 / 1.003, blue 1.004 / 1.000 (70 runs);
+//   packed half, u 1.000 / 1.000, densities 0.999 / 1.000 (70 runs).
+// So only the packed 16-bit storages fold (the rounding of the stored populations is all that counts
+// there), which takes 488 instead of 515 us a step on the 128x128x512 jet; rounding once costs FP64
+// storage 3 % of a step (32^3 55.5 -> 57.2 us) and compact storage 1.5 % (128x128x512 536 -> 545 us).
 // Relaxing the 23 moments of Eq. (momentSet) one by one between T and T^-1, with the closed forms
 // added per raw moment, took about 330 operations.  Measured with the gradients by
 // opposite pairs: collide-stream pass in FP64 on a 32^3 box (bound by the FP64 pipe) 69 -> 56 us;

@@ -33,3 +33,25 @@ def test_fp64_matches_oracle(cuda, shape, faces):
     f = lat.get_populations()
     assert np.max(np.abs(f - orc.f.reshape(f.shape))) < 1e-12 * np.max(np.abs(orc.f))
     lat.close()
+
+
+def test_fp64_rounding_no_larger_than_moment_by_moment(cuda):
+    """60 steps on eight seeded boxes: the mean distance from the oracle (2-norm, relative) is at most what
+    relaxing the 23 moments one by one shows on the same inputs, 3.57e-16 on the blue density and 7.24e-14
+    on the velocity (the folded form of the relaxation: 3.73e-16 and 7.25e-14)."""
+    err = []
+    for seed in range(1, 9):
+        p = dict(L.static_droplet(n=24, R=7.0)["params"])
+        p.update(rho_r0=1.5, nu_r=3.333e-3, nu_b=3.333e-3)
+        w = dict(name="blobs", shape=(24, 24, 24), params=p, fields=("random_blobs", dict(seed=seed, blobs=2)), steps=60)
+        rr, rb, u = L.initial_fields(w, seed=seed, u_amp=0.01)
+        lat = pkg.Lattice(w["shape"], p, storage="f64")
+        lat.init_fields(rr, rb, u)
+        lat.step(60)
+        orc = oracle.Oracle(w["shape"], p)
+        orc.init_fields(rr, rb, u)
+        orc.step(60)
+        err.append([np.linalg.norm(a - b) / np.linalg.norm(b) for a, b in zip(lat.macro(), orc.macro())])
+        lat.close()
+    _, blue, u = np.mean(err, axis=0)
+    assert blue < 3.57e-16 and u < 7.24e-14
