@@ -169,7 +169,9 @@ typedef struct {
                             differ in FP32 rounding (variant 3 also rounds the
                             densities that enter the gradients to fixed point), and
                             each is bitwise reproducible.  F32/F16/BF16 storage needs
-                            rho_r0, rho_b0 <= 64. */
+                            rho_r0, rho_b0 <= 64; under variant 3 the density of
+                            a node must stay below 1024 and its red part below
+                            512, whatever rho_r0 and rho_b0. */
   int block;             /* thread-block shape of the one-node density and
                             collide-stream kernels (variants 1 and 3, FP32
                             arithmetic): 0 = library's choice (32x2x4 for variant 3

@@ -1,5 +1,6 @@
 // Host implementation of the C ABI declared in include/lbm.h.
 #include <cuda_runtime.h>
+#include <limits.h>
 #include <math.h>
 #include <stdarg.h>
 #include <stdio.h>
@@ -44,7 +45,7 @@ struct lbm {
   void *pop, *dens, *top, *partial;
   unsigned long long* fix[2];  // fused density pass: packed fixed-point (rho, rho_r) of the state at an even / odd step
   bool fix_ready;   // fix[t & 1] holds the densities of the current state
-  long long* counter;  // [2]: step index, see k_collide_stream
+  long long* counter;  // [3]: step index, see k_collide_stream; first step with coarser fixed-point sums
   int* flag;
   double *diag_out, *scratch;
   int diag_blocks;
@@ -197,7 +198,7 @@ Layout plan(int nx, int ny, int nz, const lbm_params* p, const KernelSet* ks, in
   L.top = o;
   if (p->bc[5] == LBM_BC_OUTFLOW) o = align_up(o + (size_t)64 * align_up((size_t)Pn, 32) * ks->real_bytes, 256);
   L.counter = o;
-  o = align_up(o + 2 * sizeof(long long), 256);
+  o = align_up(o + 3 * sizeof(long long), 256);
   L.flag = o;
   o = align_up(o + sizeof(int), 256);
   L.partial = o;
@@ -255,18 +256,18 @@ lbm_status enqueue_step(lbm* h, long long t, cudaStream_t s, bool skip_density =
     LBM_CUDA(h, cudaMemsetAsync(nxt, 0, sizeof(unsigned long long) * (size_t)h->N, s));
     LBM_CUDA(h, h->ks->collide(h->pop, h->G, h->P, layout, h->dens, h->counter, h->variant, cur, nxt, h->flag,
                                h->shape, s));
-    if (outflow) LBM_CUDA(h, h->ks->outflow(h->pop, h->G, h->P, layout ^ 1, h->top, nxt, s));
+    if (outflow) LBM_CUDA(h, h->ks->outflow(h->pop, h->G, h->P, layout ^ 1, h->top, nxt, h->counter, s));
     return LBM_OK;
   }
   h->fix_ready = false;  // steps without the fused pass leave its accumulators behind
   h->launches += (skip_density ? 0 : 1) + ck + (outflow && last ? 1 : 0);
   if (!skip_density) {
     if (fold) LBM_CUDA(h, h->ks->density_fold(h->pop, h->G, h->P, layout, h->dens, h->flag, h->top, h->shape, s));
-    else LBM_CUDA(h, h->ks->density(h->pop, h->G, h->P, layout, h->dens, h->flag, nullptr, h->shape, s));
+    else LBM_CUDA(h, h->ks->density(h->pop, h->G, h->P, layout, h->dens, h->flag, nullptr, h->counter, h->shape, s));
   }
   LBM_CUDA(h, h->ks->collide(h->pop, h->G, h->P, layout, h->dens, h->counter, h->variant, nullptr, nullptr,
                              h->flag, h->shape, s));
-  if (outflow && last) LBM_CUDA(h, h->ks->outflow(h->pop, h->G, h->P, layout ^ 1, h->top, nullptr, s));
+  if (outflow && last) LBM_CUDA(h, h->ks->outflow(h->pop, h->G, h->P, layout ^ 1, h->top, nullptr, h->counter, s));
   return LBM_OK;
 }
 
@@ -285,14 +286,17 @@ lbm_status enqueue_run(lbm* h, long long t0, int n, cudaStream_t s) {
 // before fused steps from a state the fused pass did not produce: fill the accumulators of step t
 lbm_status ensure_fix(lbm* h, cudaStream_t s) {
   if (!fused_variant(h) || h->fix_ready) return LBM_OK;
-  LBM_CUDA(h, h->ks->density(h->pop, h->G, h->P, (int)(h->t & 1), h->dens, h->flag, h->fix[h->t & 1], h->shape, s));
+  LBM_CUDA(h, h->ks->density(h->pop, h->G, h->P, (int)(h->t & 1), h->dens, h->flag, h->fix[h->t & 1], h->counter,
+                             h->shape, s));
   h->fix_ready = true;
   return LBM_OK;
 }
 
-// the step index of step t for k_collide_stream
+// an uploaded state of time t: the step index for k_collide_stream (in either place), and no step yet
+// with coarser fixed-point sums
 lbm_status set_counter(lbm* h, long long t) {
-  LBM_CUDA(h, cudaMemcpyAsync(h->counter + (t & 1), &t, sizeof t, cudaMemcpyHostToDevice, h->stream));
+  const long long v[3] = {t, t, LLONG_MAX};
+  LBM_CUDA(h, cudaMemcpyAsync(h->counter, v, sizeof v, cudaMemcpyHostToDevice, h->stream));
   return LBM_OK;
 }
 
@@ -334,7 +338,8 @@ lbm_status compact_first_step(lbm* h, cudaStream_t s) {
 // compact storage: (rho, phi) of the current state in dens (pass 1, if not already there)
 lbm_status compact_dens(lbm* h) {
   if (!h->ks->compact || h->dens_ready) return LBM_OK;
-  LBM_CUDA(h, h->ks->density(h->pop, h->G, h->P, (int)(h->t & 1), h->dens, h->flag, nullptr, h->shape, h->stream));
+  LBM_CUDA(h, h->ks->density(h->pop, h->G, h->P, (int)(h->t & 1), h->dens, h->flag, nullptr, h->counter, h->shape,
+                             h->stream));
   h->dens_ready = true;
   return LBM_OK;
 }
@@ -755,14 +760,15 @@ lbm_status lbm_profile_step(lbm* h, int n, double* ms_out) {
     const size_t nfix = sizeof(unsigned long long) * (size_t)h->N;
     if (cudaEventRecord(e[0], h->stream) != cudaSuccess ||
         (fused ? cudaMemsetAsync(nxt, 0, nfix, h->stream)
-               : h->ks->density(h->pop, h->G, h->P, layout, h->dens, h->flag, nullptr, h->shape, h->stream)) !=
+               : h->ks->density(h->pop, h->G, h->P, layout, h->dens, h->flag, nullptr, h->counter, h->shape,
+                                h->stream)) !=
             cudaSuccess ||
         cudaEventRecord(e[1], h->stream) != cudaSuccess ||
         h->ks->collide(h->pop, h->G, h->P, layout, h->dens, h->counter, h->variant, fused ? cur : nullptr,
                        fused ? nxt : nullptr, h->flag, h->shape, h->stream) != cudaSuccess ||
         cudaEventRecord(e[2], h->stream) != cudaSuccess ||
-        (outflow && h->ks->outflow(h->pop, h->G, h->P, layout ^ 1, h->top, fused ? nxt : nullptr, h->stream) !=
-                        cudaSuccess) ||
+        (outflow && h->ks->outflow(h->pop, h->G, h->P, layout ^ 1, h->top, fused ? nxt : nullptr, h->counter,
+                                    h->stream) != cudaSuccess) ||
         cudaEventRecord(e[3], h->stream) != cudaSuccess) {
       st = fail(h, LBM_ECUDA, "profiled step launch: %s", cudaGetErrorString(cudaGetLastError()));
       break;
@@ -956,7 +962,7 @@ lbm_status lbm_step_pass(lbm* h, int pass) {
       LBM_CUDA(h, cudaMemsetAsync(h->fix[layout ^ 1], 0, sizeof(unsigned long long) * (size_t)h->N, s));
     } else {
       h->fix_ready = false;
-      LBM_CUDA(h, h->ks->density(h->pop, h->G, h->P, layout, h->dens, h->flag, nullptr, h->shape, s));
+      LBM_CUDA(h, h->ks->density(h->pop, h->G, h->P, layout, h->dens, h->flag, nullptr, h->counter, h->shape, s));
     }
     h->half = 1;
     return LBM_OK;
@@ -966,7 +972,8 @@ lbm_status lbm_step_pass(lbm* h, int pass) {
                              fused ? h->fix[layout] : nullptr, fused ? h->fix[layout ^ 1] : nullptr, h->flag, h->shape,
                              s));
   if (h->p.bc[5] == LBM_BC_OUTFLOW)
-    LBM_CUDA(h, h->ks->outflow(h->pop, h->G, h->P, layout ^ 1, h->top, fused ? h->fix[layout ^ 1] : nullptr, s));
+    LBM_CUDA(h, h->ks->outflow(h->pop, h->G, h->P, layout ^ 1, h->top, fused ? h->fix[layout ^ 1] : nullptr, h->counter,
+                               s));
   h->t += 1;
   h->half = 0;
   h->recs_valid = true;

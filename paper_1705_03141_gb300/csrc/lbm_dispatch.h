@@ -14,20 +14,21 @@ struct KernelSet {
   size_t dens_bytes;      // bytes per node of the pass-1 field
   size_t real_bytes;      // bytes of the compute type (outflow plane history)
   // pass 1; with fix non-null it writes the fixed-point accumulators of the fused density pass
-  // instead of dens (priming the fused pass from a stored state)
+  // instead of dens (priming the fused pass from a stored state; counter as for collide)
   // shape: block shape of the one-node kernels (0: 32x4x2, 1: 32x2x4, 2: 32x8x1; variants 1 and 3)
   cudaError_t (*density)(void* pop, const Geom& G, const Phys& P, int layout, void* dens, int* flag, void* fix,
-                         int shape, cudaStream_t s);
+                         long long* counter, int shape, cudaStream_t s);
   // pass 2.  variant: 1 = one node per thread, 2 = two nodes per thread (FP32 arithmetic, nx even),
   // 3 = one node per thread with the fused density pass (reads cur, accumulates into nxt, which
   // must be zero), 4 = software-pipelined one node per thread (packed storage), 5 = the interior
   // tiles by the TMA-pipelined kernel and the boundary tiles by variant 1 (packed storage; boxes
   // with periodic or no-slip x faces, odd nx or no interior tile run variant 1).  counter: the
-  // two-entry step index of k_collide_stream.
+  // two-entry step index of k_collide_stream and the first step with coarser fixed-point sums.
   cudaError_t (*collide)(void* pop, const Geom& G, const Phys& P, int odd, const void* dens, long long* counter,
                          int variant, const void* cur, void* nxt, int* flag, int shape, cudaStream_t s);
   // convective outflow; with fix non-null it also rewrites the top plane's accumulators
-  cudaError_t (*outflow)(void* pop, const Geom& G, const Phys& P, int layout, void* top, void* fix, cudaStream_t s);
+  cudaError_t (*outflow)(void* pop, const Geom& G, const Phys& P, int layout, void* top, void* fix,
+                         const long long* counter, cudaStream_t s);
   cudaError_t (*init)(void* pop, const Geom& G, const Phys& P, const double* rr, const double* rb, const double* u,
                       cudaStream_t s);
   cudaError_t (*get_pop)(void* pop, const Geom& G, const Phys& P, int layout, int pdir, double* out_r, double* out_b,

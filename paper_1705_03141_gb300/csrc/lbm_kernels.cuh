@@ -84,6 +84,8 @@ struct Phys {
 
 // Kernel constants in the compute type R (FP32 kernels read float constants:
 // no conversion in the inner loops).
+constexpr int kFixCoarse = 22;  // the coarsest scale of the fused density pass, 2^22
+
 template <typename R>
 struct KConst {
   R alpha_r, alpha_b;
@@ -99,6 +101,7 @@ struct KConst {
   // at red fraction q is refB[s] + q * dref[s]; dref is zero for moving classes.
   R refB[4], dref[4];
   R fix_scale, fix_inv;    // fused density pass: 2^e and 2^-e (make_kconst)
+  R fix_limit;             // density from which it goes over to 2^kFixCoarse
   // inlet (noise in FP64 so that both precisions draw the same variates)
   double rho_r0_d, alpha_r_d, u_j0, noise_frac;
   uint64_t seed;
@@ -129,12 +132,14 @@ inline KConst<R> make_kconst(const Phys& P) {
     K.dref[s] = (R)(s == 0 ? rr - rb : 0.0);  // equal for moving classes (gamma = (1-alpha_b)/(1-alpha_r))
   }
   // fixed-point densities: 2^-25 of the power of two at or above the larger phase density (the
-  // rounding of an FP32 density of that size), never coarser than 2^-22
+  // rounding of an FP32 density of that size), never coarser than 2^-kFixCoarse
   int e = 25 - (int)ceil(log2(P.rho_r0 > P.rho_b0 ? P.rho_r0 : P.rho_b0));
-  if (e < 22) e = 22;
+  if (e < kFixCoarse) e = kFixCoarse;
   if (e > 28) e = 28;
   K.fix_scale = (R)ldexp(1.0, e);
   K.fix_inv = (R)ldexp(1.0, -e);
+  // a sixteenth of the range of a partial sum, at least four times the larger phase density
+  K.fix_limit = (R)(e > kFixCoarse ? ldexp(1.0, 27 - e) : 1e30);
   K.rho_r0_d = P.rho_r0;
   K.alpha_r_d = P.alpha_r;
   K.u_j0 = P.u_j0;
@@ -724,13 +729,27 @@ __device__ __forceinline__ int tile_zmax(const Geom& G) { return G.bc[5] == BC_H
 // (boundaries: y is the owner of the slot S(x, i)), so the collide-stream
 // kernel of step t can accumulate the next step's (rho, rho_r) while it writes
 // f*, and the separate density pass (which rereads every population) is not
-// needed.  Accumulators are fixed point, value * 2^e with e = 25 for densities up to 1, 22 for
-// densities up to 64 (KConst::fix_scale): integer addition is exact and associative, so the atomics
+// needed.  Accumulators are fixed point, value * 2^e with e = 25 for phase densities up to 1, 22 for
+// those up to 64 (KConst::fix_scale): integer addition is exact and associative, so the atomics
 // of different blocks give bitwise reproducible sums in any order.  One 64-bit word per node
 // holds both, rho_r * 2^(e + 32) + rho * 2^e in two's complement: every partial sum
-// is added as one 64-bit integer, and since the total rho * 2^e lies in
-// [0, 2^32) (rho < 64 times the reference density, at least 8 times 64), the low 32 bits return rho and the
+// is added as one 64-bit integer, and while the total rho * 2^e lies in
+// [0, 2^32) and every partial sum in [-2^31, 2^31), the low 32 bits return rho and the
 // high 32 bits rho_r exactly, whatever the signs of the partial sums.
+// The fields of a run are not bound to the phase densities, so the scale follows the state: counter[2] is
+// the first step whose sums are kept with e = kFixCoarse (rho < 1024, partial sums below 512), for good.  A
+// node whose density exceeds fix_limit, a sixteenth of the range, in step t sets it to t + 1; every
+// block of a step reads the same choice, since no step sets it to itself or an earlier one.  A state
+// that enters the fused pass is converted by k_density, again where it holds such a node.
+// the sums written by step t, and those read by it (step t - 1 wrote them), for t = counter[layout of t]
+template <typename R>
+__device__ __forceinline__ R fix_scale_of(const KConst<R>& K, long long coarse, long long t) {
+  return coarse <= t ? R(1 << kFixCoarse) : K.fix_scale;
+}
+template <typename R>
+__device__ __forceinline__ R fix_inv_of(const KConst<R>& K, long long coarse, long long t) {
+  return coarse < t ? R(1.0 / (1 << kFixCoarse)) : K.fix_inv;
+}
 __device__ __forceinline__ int to_fix(float v, float scale) { return __float2int_rn(v * scale); }
 __device__ __forceinline__ unsigned long long pack_fix(float rho, float rho_r, float scale) {
   return ((unsigned long long)(unsigned)to_fix(rho_r, scale) << 32) +
@@ -741,6 +760,7 @@ struct FusedIO {
   const unsigned long long* cur;  // fixed-point (rho, rho_r) of the step's input state (index dnode)
   unsigned long long* nxt;        // accumulators of the next state (zero on entry)
   int* flag;                      // watchdog
+  float scale;                    // of the next state's accumulators
 };
 
 // (rho, phi) of a density-tile cell from the fixed-point accumulators; the
@@ -815,8 +835,8 @@ __device__ __forceinline__ void axis_target(int& q, int p, int c, int n, int bc_
 // (bounced back to x, reflected, wrapped, or into the ghost plane above an
 // outflow face, which no node reads as a density).
 template <int T, typename R>
-__device__ __forceinline__ void fused_node(const Geom& G, const FusedIO& io, R scale, int x, int y, int z,
-                                           const R f[27], const Recol<R>& rc) {
+__device__ __forceinline__ void fused_node(const Geom& G, const FusedIO& io, int x, int y, int z, const R f[27],
+                                           const Recol<R>& rc) {
   constexpr int dx = cx_of(T), dy = cy_of(T), dz = cz_of(T);
   int tx = x + dx, ty = y + dy, tz = z + dz;
   bool bounce = false, ghost = false;
@@ -830,7 +850,7 @@ __device__ __forceinline__ void fused_node(const Geom& G, const FusedIO& io, R s
   } else if (ghost) {
     return;
   }
-  atomicAdd(io.nxt + dnode(G, tx, ty, tz), pack_fix((float)f[T], (float)red_part<T, true>(f[T], rc), scale));
+  atomicAdd(io.nxt + dnode(G, tx, ty, tz), pack_fix((float)f[T], (float)red_part<T, true>(f[T], rc), io.scale));
 }
 
 // grad phi and grad rho at tile cell (lx, ly, lz) from the (rho, phi) halo tile:
@@ -952,7 +972,7 @@ struct EmitLoop {
       if constexpr (FAST) {
         if constexpr (T % 3 == 2) fused_row<T / 3, RECOL, R, BYv, TXv>(prow, min(31, G.nx - 1 - (x - (int)threadIdx.x)), f, rc);
       } else {
-        fused_node<T>(G, io, (R)K.fix_scale, x, y, z, f, rc);
+        fused_node<T>(G, io, x, y, z, f, rc);
       }
     }
     EmitLoop<T + 1, Store, R, FAST, RECOL, FUSED, ODDT, BYv, TXv>::run(st, K, G, nm, ar, odd, f, rc, prow, io, x, y, z);
@@ -1104,14 +1124,20 @@ __device__ __forceinline__ V density_value(const KConst<D>& K, D rr, const D ft[
 // the steps of a run; the blocks of the top planes start first (z blocks in reverse order).
 // Four blocks per SM (64 registers): the outflow path of the top plane may spill, the pass over
 // the rest of the box keeps its occupancy (a streaming pass, bound by memory parallelism).
+// FIX: into the accumulators of the fused pass (a second launch, again != 0, writes them coarser where
+// the first one met a density beyond fix_limit).
 template <class Store, bool FIX, class B = BlkDefault>
 __global__ void __launch_bounds__(B::NT, 4) k_density(Store st, Geom G,
                                                       const __grid_constant__ KConst<typename DensOf<Store>::real> K,
                                                       int layout, typename DensOf<Store>::type* __restrict__ dens,
                                                       int* __restrict__ flag,
                                                       unsigned long long* __restrict__ fix,
-                                                      typename DensOf<Store>::real* __restrict__ top) {
+                                                      typename DensOf<Store>::real* __restrict__ top,
+                                                      long long* counter, int again) {
   using D = typename DensOf<Store>::real;
+  // the sums of time t = counter[layout], as step t - 1 would have written them
+  const long long t = FIX ? counter[layout] : 0, coarse = FIX ? counter[2] : 0;
+  if (FIX && again && coarse >= t) return;
   const int x = blockIdx.x * B::BX + threadIdx.x;
   const int y = blockIdx.y * B::BY + threadIdx.y;
   const int z = (gridDim.z - 1 - face_first(blockIdx.z, gridDim.z, G.bc[4])) * B::BZ + threadIdx.z;
@@ -1135,7 +1161,8 @@ __global__ void __launch_bounds__(B::NT, 4) k_density(Store st, Geom G,
 #pragma unroll
     for (int t = 0; t < 27; ++t) rt += ft[t];
     if (!(rt > D(0)) || !(rt < D(1e30))) atomicOr(flag, 1);
-    fix[dnode(G, x, y, z)] = pack_fix((float)rt, (float)rr, (float)K.fix_scale);
+    if (rt > (D)K.fix_limit && coarse >= t) atomicMin(counter + 2, t - 1);
+    fix[dnode(G, x, y, z)] = pack_fix((float)rt, (float)rr, (float)fix_scale_of(K, coarse, t - 1));
   } else {
     dens[dnode(G, x, y, z)] = density_value<D, typename DensOf<Store>::type>(K, rr, ft, is_inlet(G, x, y, z), flag);
   }
@@ -1304,6 +1331,8 @@ __global__ void __launch_bounds__(B::NT, MINB)
   const int tid = threadIdx.x + B::BX * (threadIdx.y + B::BY * threadIdx.z);
   const long long step = counter[odd];
   if (tid == 0 && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0) counter[odd ^ 1] = step + 1;
+  const long long coarse = FUSED ? counter[2] : 0;
+  const R fix_inv = FUSED ? fix_inv_of(K, coarse, step) : R(0), fix_scale = FUSED ? fix_scale_of(K, coarse, step) : R(0);
 
   // block-uniform: the tile comes by TMA (no periodic face crossed)
   bool via_tma = false;
@@ -1369,8 +1398,8 @@ __global__ void __launch_bounds__(B::NT, MINB)
         const int cy = gy < G.ny ? gy : G.ny - 1, cz = gz <= tile_zmax(G) ? gz : tile_zmax(G);
         const int64_t rbase = (int64_t)G.nx * ((int64_t)cy + (int64_t)G.ny * cz);
         if constexpr (FUSED) {
-          tile[row * B::TXT + 1 + lane] = fused_cell(io, rbase + cxa, K.fix_inv);
-          if (lane < B::TX - 32) tile[row * B::TXT + 33 + lane] = fused_cell(io, rbase + cxb, K.fix_inv);
+          tile[row * B::TXT + 1 + lane] = fused_cell(io, rbase + cxa, fix_inv);
+          if (lane < B::TX - 32) tile[row * B::TXT + 33 + lane] = fused_cell(io, rbase + cxb, fix_inv);
         } else {
           tile[row * B::TXT + 1 + lane] = dens[rbase + cxa];
           if (lane < B::TX - 32) tile[row * B::TXT + 33 + lane] = dens[rbase + cxb];
@@ -1419,30 +1448,33 @@ __global__ void __launch_bounds__(B::NT, MINB)
     if constexpr (FUSED) {
       // the watchdog of pass 1, on the density this step starts from
       if (!(rc.rho > R(0)) || !(rc.rho < R(1e30))) atomicOr(io.flag, 1);
+      if (rc.rho > K.fix_limit && coarse > step + 1) atomicMin(counter + 2, step + 1);
     }
     // warp-uniform: does any node of the warp carry an interface normal?
     const bool recol = __any_sync(__activemask(), any_(rc.has_n));
     NodeMap nm;
     AoRow ar;
+    FusedIO fio = io;
+    if constexpr (FUSED) fio.scale = fix_scale;
     if (fast) {
       ar.init<Store::PLANES>(G, x, y, z);
       // the parity as a template argument: no per-direction branch on it in the stores (the
       // fused density pass keeps it a runtime value: the extra code raised its spills)
       if constexpr (FUSED) {
-        if (recol) EmitLoop<0, Store, R, true, true, FUSED, -1, B::BY, B::TX>::run(st, K, G, nm, ar, odd != 0, f, rc, prow, io, x, y, z);
-        else EmitLoop<0, Store, R, true, false, FUSED, -1, B::BY, B::TX>::run(st, K, G, nm, ar, odd != 0, f, rc, prow, io, x, y, z);
+        if (recol) EmitLoop<0, Store, R, true, true, FUSED, -1, B::BY, B::TX>::run(st, K, G, nm, ar, odd != 0, f, rc, prow, fio, x, y, z);
+        else EmitLoop<0, Store, R, true, false, FUSED, -1, B::BY, B::TX>::run(st, K, G, nm, ar, odd != 0, f, rc, prow, fio, x, y, z);
       } else if (recol) {
-        if (odd) EmitLoop<0, Store, R, true, true, FUSED, 1, B::BY, B::TX>::run(st, K, G, nm, ar, true, f, rc, prow, io, x, y, z);
-        else EmitLoop<0, Store, R, true, true, FUSED, 0, B::BY, B::TX>::run(st, K, G, nm, ar, false, f, rc, prow, io, x, y, z);
+        if (odd) EmitLoop<0, Store, R, true, true, FUSED, 1, B::BY, B::TX>::run(st, K, G, nm, ar, true, f, rc, prow, fio, x, y, z);
+        else EmitLoop<0, Store, R, true, true, FUSED, 0, B::BY, B::TX>::run(st, K, G, nm, ar, false, f, rc, prow, fio, x, y, z);
       } else {
-        if (odd) EmitLoop<0, Store, R, true, false, FUSED, 1, B::BY, B::TX>::run(st, K, G, nm, ar, true, f, rc, prow, io, x, y, z);
-        else EmitLoop<0, Store, R, true, false, FUSED, 0, B::BY, B::TX>::run(st, K, G, nm, ar, false, f, rc, prow, io, x, y, z);
+        if (odd) EmitLoop<0, Store, R, true, false, FUSED, 1, B::BY, B::TX>::run(st, K, G, nm, ar, true, f, rc, prow, fio, x, y, z);
+        else EmitLoop<0, Store, R, true, false, FUSED, 0, B::BY, B::TX>::run(st, K, G, nm, ar, false, f, rc, prow, fio, x, y, z);
       }
     } else {
       if (odd) nm.init(G, x, y, z);
       else nm.base = snode(G, x, y, z);  // the even step only uses the base
-      if (recol) EmitLoop<0, Store, R, false, true, FUSED, -1, B::BY, B::TX>::run(st, K, G, nm, ar, odd != 0, f, rc, prow, io, x, y, z);
-      else EmitLoop<0, Store, R, false, false, FUSED, -1, B::BY, B::TX>::run(st, K, G, nm, ar, odd != 0, f, rc, prow, io, x, y, z);
+      if (recol) EmitLoop<0, Store, R, false, true, FUSED, -1, B::BY, B::TX>::run(st, K, G, nm, ar, odd != 0, f, rc, prow, fio, x, y, z);
+      else EmitLoop<0, Store, R, false, false, FUSED, -1, B::BY, B::TX>::run(st, K, G, nm, ar, odd != 0, f, rc, prow, fio, x, y, z);
     }
   }
 
@@ -1495,7 +1527,7 @@ __global__ void __launch_bounds__(B::NT, MINB)
             }
           }
           const int64_t rb = (int64_t)G.nx * ((int64_t)gy + (int64_t)G.ny * gz);
-          const unsigned long long av = pack_fix(a.x, a.y, K.fix_scale), bv = pack_fix(b.x, b.y, K.fix_scale);
+          const unsigned long long av = pack_fix(a.x, a.y, fix_scale), bv = pack_fix(b.x, b.y, fix_scale);
           if (ina && av) atomicAdd(io.nxt + rb + gxa, av);
           if (inb && bv) atomicAdd(io.nxt + rb + gxb, bv);
         }
@@ -2020,7 +2052,8 @@ template <class Store>
 __global__ void __launch_bounds__(32 * OUT_W)
     k_outflow(Store st, const __grid_constant__ Geom G,
               const __grid_constant__ KConst<typename DensOf<Store>::real> K, int layout,
-              typename DensOf<Store>::real* __restrict__ top, unsigned long long* __restrict__ fix) {
+              typename DensOf<Store>::real* __restrict__ top, unsigned long long* __restrict__ fix,
+              const long long* __restrict__ counter) {
   using R = typename DensOf<Store>::real;
   __shared__ OutflowSums<R> sh, shf;
   int x, y;
@@ -2056,7 +2089,9 @@ __global__ void __launch_bounds__(32 * OUT_W)
     if (in && threadIdx.y == 0) {
       R rho, rr;
       outflow_total(shf, rho, rr);
-      fix[dnode(G, x, y, G.nz - 1)] = pack_fix((float)rho, (float)rr, (float)K.fix_scale);
+      // as the step before wrote the others: counter[layout] is its index plus one
+      const float scale = (float)fix_scale_of(K, counter[2], counter[layout] - 1);
+      fix[dnode(G, x, y, G.nz - 1)] = pack_fix((float)rho, (float)rr, scale);
     }
   }
 }

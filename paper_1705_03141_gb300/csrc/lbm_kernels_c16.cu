@@ -48,7 +48,7 @@ struct LaunchCompact {
   // pass 1: shape 3 the TMA pipeline (k_density_ct; x faces that reflect and at least 3 tiles along
   // y and z, checked at creation), otherwise one block per 32x4x2 tile
   static cudaError_t density(void* pop, const Geom& G, const Phys& P, int layout, void* dens, int* flag, void*,
-                             int shape, cudaStream_t s) {
+                             long long*, int shape, cudaStream_t s) {
     const Store st = make(pop, G);
     if (shape != 3) {
       k_density_c<B><<<grid3(G), dim3(BX, BY, BZ), 0, s>>>(st, G, kc(P), layout, static_cast<float2*>(dens), flag);
@@ -77,7 +77,7 @@ struct LaunchCompact {
                                                                  static_cast<const float2*>(dens), counter);
     return cudaGetLastError();
   }
-  static cudaError_t outflow(void* pop, const Geom& G, const Phys& P, int layout, void*, void*, cudaStream_t s) {
+  static cudaError_t outflow(void* pop, const Geom& G, const Phys& P, int layout, void*, void*, const long long*, cudaStream_t s) {
     k_outflow_c<B><<<outflow_grid(G), outflow_block(), 0, s>>>(
         make(pop, G), G, kc(P), layout);
     return cudaGetLastError();

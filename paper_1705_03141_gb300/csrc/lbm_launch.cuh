@@ -53,39 +53,40 @@ struct Launch {
 
   template <class B>
   static cudaError_t density_b(void* pop, const Geom& G, const Phys& P, int layout, void* dens, int* flag, void* fix,
-                               void* top, cudaStream_t s) {
+                               void* top, long long* counter, cudaStream_t s) {
     if constexpr (fused) {
       if (fix) {
-        k_density<Store, true, B><<<grid3<B>(G), dim3(B::BX, B::BY, B::BZ), 0, s>>>(
-            Tr::make(pop, G), G, kc(P), layout, static_cast<DT*>(dens), flag, static_cast<unsigned long long*>(fix),
-            nullptr);
+        for (int again = 0; again < 2; ++again)
+          k_density<Store, true, B><<<grid3<B>(G), dim3(B::BX, B::BY, B::BZ), 0, s>>>(
+              Tr::make(pop, G), G, kc(P), layout, static_cast<DT*>(dens), flag, static_cast<unsigned long long*>(fix),
+              nullptr, counter, again);
         return cudaGetLastError();
       }
     }
     k_density<Store, false, B><<<grid3<B>(G), dim3(B::BX, B::BY, B::BZ), 0, s>>>(
-        Tr::make(pop, G), G, kc(P), layout, static_cast<DT*>(dens), flag, nullptr, static_cast<R*>(top));
+        Tr::make(pop, G), G, kc(P), layout, static_cast<DT*>(dens), flag, nullptr, static_cast<R*>(top), nullptr, 0);
     return cudaGetLastError();
   }
   static cudaError_t density_top(void* pop, const Geom& G, const Phys& P, int layout, void* dens, int* flag,
-                                 void* fix, void* top, int shape, cudaStream_t s) {
+                                 void* fix, void* top, int shape, long long* counter, cudaStream_t s) {
     if constexpr (std::is_same<R, double>::value) {  // node after node: no blocks of rows
       k_density_lin<Store><<<blocks1((int64_t)G.nx * G.ny * G.nz, LIN_THREADS), LIN_THREADS, 0, s>>>(
           Tr::make(pop, G), G, kc(P), layout, static_cast<DT*>(dens), flag, static_cast<R*>(top));
       return cudaGetLastError();
     } else {
-      if (shape == 1) return density_b<Blk<2, 4>>(pop, G, P, layout, dens, flag, fix, top, s);
-      if (shape == 2) return density_b<Blk<8, 1>>(pop, G, P, layout, dens, flag, fix, top, s);
-      return density_b<BlkDefault>(pop, G, P, layout, dens, flag, fix, top, s);
+      if (shape == 1) return density_b<Blk<2, 4>>(pop, G, P, layout, dens, flag, fix, top, counter, s);
+      if (shape == 2) return density_b<Blk<8, 1>>(pop, G, P, layout, dens, flag, fix, top, counter, s);
+      return density_b<BlkDefault>(pop, G, P, layout, dens, flag, fix, top, counter, s);
     }
   }
   static cudaError_t density(void* pop, const Geom& G, const Phys& P, int layout, void* dens, int* flag, void* fix,
-                             int shape, cudaStream_t s) {
-    return density_top(pop, G, P, layout, dens, flag, fix, nullptr, shape, s);
+                             long long* counter, int shape, cudaStream_t s) {
+    return density_top(pop, G, P, layout, dens, flag, fix, nullptr, shape, counter, s);
   }
   // pass 1 of a step that first completes the step before with its convective outflow
   static cudaError_t density_fold(void* pop, const Geom& G, const Phys& P, int layout, void* dens, int* flag,
                                   void* top, int shape, cudaStream_t s) {
-    return density_top(pop, G, P, layout, dens, flag, nullptr, top, shape, s);
+    return density_top(pop, G, P, layout, dens, flag, nullptr, top, shape, nullptr, s);
   }
   // Tensor map of the pass-1 field for the TMA tile of k_collide_stream: 8-byte cells (rho, phi)
   // over (x, y, z + 1), planes z = -1 .. nz (dens points at plane 0, one plane above the start of
@@ -212,9 +213,9 @@ struct Launch {
     }
   }
   static cudaError_t outflow(void* pop, const Geom& G, const Phys& P, int layout, void* top, void* fix,
-                             cudaStream_t s) {
+                             const long long* counter, cudaStream_t s) {
     k_outflow<Store><<<outflow_grid(G), outflow_block(), 0, s>>>(
-        Tr::make(pop, G), G, kc(P), layout, static_cast<R*>(top), static_cast<unsigned long long*>(fix));
+        Tr::make(pop, G), G, kc(P), layout, static_cast<R*>(top), static_cast<unsigned long long*>(fix), counter);
     return cudaGetLastError();
   }
   static cudaError_t init(void* pop, const Geom& G, const Phys& P, const double* rr, const double* rb, const double* u,

@@ -149,7 +149,7 @@ def test_two_node_kernel_needs_even_nx(lib):
 
 
 def test_fixed_point_range_checked_for_fp32_storages(lib):
-    """The fused pass keeps densities in 2^-22 fixed point: FP32/packed storage rejects rho0 > 64."""
+    """The fused pass keeps densities in fixed point, 2^-22 at its coarsest: FP32/packed storage rejects rho0 > 64."""
     w = L.static_droplet(n=8, R=2.0)
     params = {**w["params"], "rho_r0": 80.0, "rho_b0": 40.0}
     assert _size(lib, w["shape"], params, 1)[0] == -1

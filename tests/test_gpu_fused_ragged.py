@@ -53,6 +53,46 @@ def test_fused_ragged_rows(cuda, shape, faces):
         assert np.array_equal(x, y)  # bitwise reproducible
 
 
+# densities far from the phase densities, which set the scale of the fixed-point sums: beyond the fine
+# scale's range from the start (times 200), and growing past the density at which the scale changes
+# on the way (phase densities 0.05: 2^-28 up to 0.5, range 8; the fields reach 0.36 at first, 0.58 later)
+@pytest.mark.parametrize("faces", ["periodic", "walls", "jet"])
+@pytest.mark.parametrize("ref,amp", [(1.0, 200.0), (0.05, 0.3)])
+def test_fused_density_range(cuda, faces, ref, amp):
+    shape = (34, 20, 18)
+    w = _work(shape, faces)
+    p = w["params"]
+    p.update(rho_r0=ref, rho_b0=ref, A=0.0, beta=0.0)
+    if faces == "jet":
+        p["inflow"].update(D=1.0, u_j0=0.0, noise_frac=0.0)  # one inlet node
+    x = np.arange(shape[0])[None, None, :] + 0.5
+    z = np.arange(shape[2])[:, None, None] + 0.5
+    one = np.ones((shape[2], shape[1], shape[0]))
+    rho = amp * (1.0 + 0.2 * np.cos(2 * np.pi * x / shape[0])) * one
+    q = 0.5 + 0.3 * np.cos(2 * np.pi * z / shape[2])
+    u = np.zeros((3,) + rho.shape)
+    u[0] = 0.3 * np.sin(2 * np.pi * x / shape[0]) * one  # towards the middle of the box
+    peak = []
+
+    def run(variant, chunks):
+        lat = pkg.Lattice(shape, p, storage="f32", variant=variant)
+        lat.init_fields(q * rho, (1 - q) * rho, u)
+        for n in chunks:
+            lat.step(n)
+            peak.append(max(np.max(np.add(*lat.macro()[:2])), 0))
+        f, m = lat.get_populations(), lat.macro()
+        lat.close()
+        return f, m
+
+    f1, (r1, b1, u1) = run(1, (8, 16, 16))
+    print(faces, ref, "largest density", peak)
+    for chunks in ((8, 16, 16), (1,) * 8 + (32,)):
+        f3, (r, b, v) = run(3, chunks)
+        scale = np.max(np.abs(r1) + np.abs(b1))
+        assert np.max(np.abs(r - r1)) < 2e-5 * scale and np.max(np.abs(b - b1)) < 2e-5 * scale
+        assert np.max(np.abs(v - u1)) < 1e-4 * np.max(np.abs(u1)) + 3e-6
+
+
 def test_library_choice_by_size(cuda):
     for shape, faces, variant in (((64, 20, 40), "periodic", 3), ((66, 20, 40), "periodic", 1),
                                   ((126, 104, 41), "periodic", 3), ((66, 20, 40), "jet", 3),
