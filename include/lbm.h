@@ -144,9 +144,10 @@ typedef struct {
                             allocates (cudaMalloc) and frees it itself. */
   size_t workspace_bytes;
   int variant;           /* collide-stream kernel: 0 = library's choice (3 for F32
-                            storage with nx a multiple of 32 or, by size, where
-                            it is faster, 5 for F16/BF16 storage, 1 otherwise: the
-                            measured faster ones; slab handles 1 for F32),
+                            storage where no x face is no-slip and nx is a
+                            multiple of 32 or the size makes it faster, 5 for
+                            F16/BF16 storage, 1 otherwise: the measured faster
+                            ones; slab handles 1 for F32),
                             1 = one node per thread, 2 = two x-adjacent nodes per
                             thread with packed FP32x2 arithmetic (needs F32/F16/BF16
                             storage and an even nx), 3 = one node per thread with

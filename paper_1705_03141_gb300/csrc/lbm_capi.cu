@@ -106,17 +106,22 @@ bool pipelined_ok(int nx, int ny, int nz, const lbm_params* p) {
          p->bc[1] != LBM_BC_NOSLIP && nx % 32 != 1 && ny > 2 * lbmk::BY && nz > 2 * lbmk::BZ;
 }
 
-// where FP32 storage runs the fused density pass: its collide-stream kernel is bound by memory, so
+// where FP32 storage runs the fused density pass.  Not with no-slip x faces: no row is a fast row then, and
+// every population goes to the accumulators by its own atomic; us a step, fused / two passes: 64^3
+// 44.4 / 33.3, 85^3 123 / 91, 128^3 338 / 252, 33x128x128 179 / 129, 64x64x256 jet 189 / 126, 66x20x40 jet
+// 26.5 / 24.6.  Elsewhere its collide-stream kernel is bound by memory, so
 // that dropping pass 1 pays, always where rows fill whole 32-node blocks.  Ragged rows leave lanes of the
 // (longer) fused kernel idle, and pass 1 finds much of a small box in L2, so there it depends on the
 // size; us a step, fused / two passes, no outflow face: 41^3 15.1 / 14.5, 60^3 26.2 / 24.9, 70^3 47.7 /
-// 47.0, 75^3 55.6 / 57.6, 80^3 59.2 / 63.0, 85^3 70.4 / 77.0, 97^3 121 / 128, 120^3 170 / 191.  An outflow face adds
+// 47.0, 75^3 55.6 / 57.6, 80^3 59.2 / 63.0, 85^3 70.4 / 77.0, 97^3 121 / 128, 120^3 170 / 191; the emptiest last
+// blocks, 33x110x110 74.7 / 77.8, 33x200x200 246 / 272, 36x128x128 105 / 107, 65x80x80 60.4 / 62.7.  An outflow face adds
 // the outflow kernel to each fused step, while the two passes fold it into pass 1, where it is the
 // tail on small boxes: 66x20x40 14.8 / 18.4, 50x50x100 36.4 / 38.7, 90x90x120 121 / 111,
 // 110x100x100 143 / 134, 120^3 180 / 187, 100x100x200 265 / 277, 200x200x500 2048 / 2277.
-bool fused_pays(int nx, int64_t N, bool outflow) {
+bool fused_pays(int nx, int64_t N, const lbm_params* p) {
+  if (p->bc[0] == LBM_BC_NOSLIP || p->bc[1] == LBM_BC_NOSLIP) return false;
   if (nx % 32 == 0) return true;
-  return outflow ? N < (1 << 18) || N >= (3 << 19) : N >= (3 << 17);
+  return p->bc[5] == LBM_BC_OUTFLOW ? N < (1 << 18) || N >= (3 << 19) : N >= (3 << 17);
 }
 
 const char* validate(int nx, int ny, int nz, const lbm_params* p) {
@@ -410,7 +415,7 @@ lbm_status lbm_create(int nx, int ny, int nz, const lbm_params* p, lbm** out) {
   h->dens_ready = false;
   const bool packed = p->storage == LBM_STORE_F16 || p->storage == LBM_STORE_BF16;
   h->variant = p->variant != 0 ? p->variant
-                               : (p->storage == LBM_STORE_F32 && !h->halo && fused_pays(nx, h->N, p->bc[5] == LBM_BC_OUTFLOW)
+                               : (p->storage == LBM_STORE_F32 && !h->halo && fused_pays(nx, h->N, p)
                                       ? 3
                                       : (packed ? 5 : 1));
   h->fix_ready = false;

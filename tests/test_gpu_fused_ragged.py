@@ -14,9 +14,10 @@ import paper_1705_03141_gb300 as pkg
 
 pytestmark = pytest.mark.gpu
 
-# last block with 1, 2 and 31 nodes, less than one block, whole blocks; every x face that has fast rows
+# last block with 1, 2 and 31 nodes, less than one block, whole blocks; x faces with fast rows and without
 SHAPES = [(33, 8, 9), (34, 9, 8), (63, 7, 10), (21, 12, 9), (64, 8, 8)]
-FACES = {"periodic": (0, 0, 0, 0, 0, 0), "jet": (2, 2, 2, 2, 3, 4), "walls": (2, 2, 1, 1, 1, 1)}
+FACES = {"periodic": (0, 0, 0, 0, 0, 0), "jet": (2, 2, 2, 2, 3, 4), "walls": (2, 2, 1, 1, 1, 1),
+         "no-slip x": (1, 1, 0, 0, 0, 0), "one no-slip x": (1, 2, 2, 2, 2, 2)}
 
 
 def _work(shape, faces):
@@ -96,7 +97,9 @@ def test_fused_density_range(cuda, faces, ref, amp):
 def test_library_choice_by_size(cuda):
     for shape, faces, variant in (((64, 20, 40), "periodic", 3), ((66, 20, 40), "periodic", 1),
                                   ((126, 104, 41), "periodic", 3), ((66, 20, 40), "jet", 3),
-                                  ((126, 104, 41), "jet", 1), ((126, 104, 121), "jet", 3)):
+                                  ((126, 104, 41), "jet", 1), ((126, 104, 121), "jet", 3),
+                                  ((64, 20, 40), "no-slip x", 1), ((126, 104, 41), "no-slip x", 1),
+                                  ((96, 9, 8), "one no-slip x", 1)):
         lat = pkg.Lattice(shape, _work(shape, faces)["params"], storage="f32")
         assert lat.variant == variant
         lat.close()
