@@ -85,6 +85,12 @@ struct Phys {
 // Kernel constants in the compute type R (FP32 kernels read float constants:
 // no conversion in the inner loops).
 constexpr int kFixCoarse = 22;  // the coarsest scale of the fused density pass, 2^22
+// its scale 2^e: 2^-25 of the power of two at or above the larger phase density (the rounding of an FP32
+// density of that size), never coarser than 2^-kFixCoarse
+inline int fix_exponent(double rho_r0, double rho_b0) {
+  const int e = 25 - (int)ceil(log2(rho_r0 > rho_b0 ? rho_r0 : rho_b0));
+  return e < kFixCoarse ? kFixCoarse : (e > 28 ? 28 : e);
+}
 
 template <typename R>
 struct KConst {
@@ -131,11 +137,7 @@ inline KConst<R> make_kconst(const Phys& P) {
     K.refB[s] = (R)rb;
     K.dref[s] = (R)(s == 0 ? rr - rb : 0.0);  // equal for moving classes (gamma = (1-alpha_b)/(1-alpha_r))
   }
-  // fixed-point densities: 2^-25 of the power of two at or above the larger phase density (the
-  // rounding of an FP32 density of that size), never coarser than 2^-kFixCoarse
-  int e = 25 - (int)ceil(log2(P.rho_r0 > P.rho_b0 ? P.rho_r0 : P.rho_b0));
-  if (e < kFixCoarse) e = kFixCoarse;
-  if (e > 28) e = 28;
+  const int e = fix_exponent(P.rho_r0, P.rho_b0);
   K.fix_scale = (R)ldexp(1.0, e);
   K.fix_inv = (R)ldexp(1.0, -e);
   // a sixteenth of the range of a partial sum, at least four times the larger phase density

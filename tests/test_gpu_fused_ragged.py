@@ -103,3 +103,11 @@ def test_library_choice_by_size(cuda):
         lat = pkg.Lattice(shape, _work(shape, faces)["params"], storage="f32")
         assert lat.variant == variant
         lat.close()
+    # a light phase with fewer than 23 bits above the fixed-point step: two passes on ragged rows
+    for rho, shape, variant in (((4.0, 1.0), (126, 104, 41), 3), ((8.0, 1.0), (126, 104, 41), 1),
+                                ((1.0, 0.1), (126, 104, 41), 1), ((0.1, 0.1), (126, 104, 41), 3),
+                                ((1e-3, 1e-3), (126, 104, 41), 1), ((8.0, 1.0), (64, 20, 40), 3)):
+        p = dict(_work(shape, "periodic")["params"], rho_r0=rho[0], rho_b0=rho[1])
+        lat = pkg.Lattice(shape, p, storage="f32")
+        assert lat.variant == variant, rho
+        lat.close()
