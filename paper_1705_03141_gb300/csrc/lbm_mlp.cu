@@ -24,6 +24,7 @@
 #include <vector>
 
 #include "../../include/lbm_mlp.h"
+#include "lbm_mlp_buffers.h"
 
 namespace {
 
@@ -803,6 +804,7 @@ unsigned blocks(long long n, int t) { return (unsigned)((n + t - 1) / t); }
 
 struct lbm_mlp {
   int n_in, width, depth, n_pos, n_cls, n_out, max_batch;
+  int device;
   cudaStream_t stream;
   std::vector<int> fan_in, fan_out;  // per layer
   std::vector<size_t> w_off, b_off;  // flat offsets
@@ -943,23 +945,41 @@ lbm_status stage_inputs(lbm_mlp* m, const float* x, const float* target, const i
   return LBM_OK;
 }
 
-// device pointer of an input: the caller's own where it is device memory, else a copy at `staged`
+// may the kernels use the caller's buffer itself
+bool in_place(const lbm_mlp* m, const void* ptr) {
+  cudaPointerAttributes a;
+  if (!ptr) return false;
+  if (cudaPointerGetAttributes(&a, ptr) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return mlpbuf::in_place(a.type == cudaMemoryTypeDevice, a.type == cudaMemoryTypeManaged, a.device, m->device,
+                          reinterpret_cast<uintptr_t>(ptr));
+}
+
+// device pointer of an input: the caller's own where the kernels may use it and it stays as it is while
+// they run, else a copy at `staged`
 template <typename V>
-lbm_status on_device(lbm_mlp* m, const V* src, V* staged, size_t n, const V** out) {
-  if (is_device_ptr(src)) {
+lbm_status on_device(lbm_mlp* m, const V* src, V* staged, size_t n, const V** out, bool stays = true) {
+  if (stays && in_place(m, src)) {
     *out = src;
     return LBM_OK;
   }
-  MLP_CUDA(cudaMemcpyAsync(staged, src, sizeof(V) * n, cudaMemcpyHostToDevice, m->stream));
+  const cudaMemcpyKind k = is_device_ptr(src) ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
+  MLP_CUDA(cudaMemcpyAsync(staged, src, sizeof(V) * n, k, m->stream));
   *out = staged;
   return LBM_OK;
 }
 
-// fused forward pass; y: device memory
+// fused forward pass; y: memory that the kernels may use.  An x that y overlaps is staged: a block
+// writes the outputs of its rows while others have yet to read theirs.
 lbm_status fused_forward(lbm_mlp* m, const float* x, int batch, float* y) {
   RowsArgs A;
   memset(&A, 0, sizeof A);
-  lbm_status st = on_device(m, x, m->x32, (size_t)batch * m->n_in, &A.x);
+  const size_t nx = (size_t)batch * m->n_in, ny = (size_t)batch * m->n_out;
+  const bool apart = !mlpbuf::overlap(reinterpret_cast<uintptr_t>(x), sizeof(float) * nx,
+                                      reinterpret_cast<uintptr_t>(y), sizeof(float) * ny);
+  lbm_status st = on_device(m, x, m->x32, nx, &A.x, apart);
   if (st != LBM_OK) return st;
   A.y = y;
   A.p = m->p;
@@ -1074,6 +1094,11 @@ lbm_status lbm_mlp_create(int n_in, int width, int depth, int n_pos, int n_cls, 
   m->max_batch = max_batch;
   m->stream = static_cast<cudaStream_t>(cuda_stream);
   m->step = 0;
+  if (cudaGetDevice(&m->device) != cudaSuccess) {
+    cudaGetLastError();
+    delete m;
+    return LBM_ECUDA;
+  }
   const int L = depth + 1;
   size_t o = 0;
   for (int l = 0; l < L; ++l) {
@@ -1217,9 +1242,9 @@ lbm_status lbm_mlp_forward(lbm_mlp* m, const float* x, int batch, float* y) {
   if (!m || !x || !y || batch < 1 || batch > m->max_batch) return LBM_EINVAL;
   lbm_status st;
   if (m->fused) {
-    const bool dev = is_device_ptr(y);  // the answers go straight to the caller's device memory
-    st = fused_forward(m, x, batch, dev ? y : m->y);
-    if (st == LBM_OK && !dev) st = copy_out(m, y, m->y, sizeof(float) * batch * m->n_out);
+    const bool own = in_place(m, y);  // the answers go straight to the caller's device memory
+    st = fused_forward(m, x, batch, own ? y : m->y);
+    if (st == LBM_OK && !own) st = copy_out(m, y, m->y, sizeof(float) * batch * m->n_out);
   } else {
     st = stage_inputs(m, x, nullptr, nullptr, batch);
     if (st == LBM_OK) st = forward(m, batch);

@@ -94,3 +94,21 @@ def test_forward_gradient_and_step(cuda, n_in, width, depth, n_pos, n_cls, batch
         assert net.loss_grad(x, t, lab)[0] == la
     net.close()
     fresh.close()
+
+
+# n_in, n_out and batch of more than one block, y ahead of, at and behind the start of x
+@pytest.mark.parametrize("offset", [-340, -5, 0, 5, 340])
+@pytest.mark.parametrize("n_in,n_out,batch", [(5, 68, 4096), (40, 4, 3000), (8, 8, 333)])
+def test_output_overlapping_the_input(cuda, n_in, n_out, batch, offset):
+    import torch
+
+    net = pkg.Mlp(n_in=n_in, width=128, depth=2, n_pos=n_out, n_cls=0, max_batch=batch, seed=3)
+    x = torch.rand(batch, n_in, generator=torch.Generator().manual_seed(1)).cuda()
+    want = net.forward(x)
+    buf = torch.zeros(512 + batch * max(n_in, n_out) + 512, device="cuda")
+    xv = buf[512:512 + batch * n_in].view(batch, n_in)
+    xv.copy_(x)
+    yv = buf[512 + offset:512 + offset + batch * n_out].view(batch, n_out)
+    got = net.forward(xv, out=yv)
+    assert got.data_ptr() == yv.data_ptr() and torch.equal(got, want)
+    net.close()
