@@ -772,12 +772,17 @@ constexpr size_t STAGE_BYTES = 128 * 1024;
 
 template <int MT, bool TRAIN>
 cudaError_t launch_rows_mt(const NetShape& S, const RowsArgs& A, cudaStream_t s) {
-  const size_t smem = rows_smem<TRAIN>(S, MT);
-  static const cudaError_t attr =
-      cudaFuncSetAttribute(k_rows<MT, TRAIN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ROWS_SMEM_MAX);
-  if (attr != cudaSuccess) return attr;
-  k_rows<MT, TRAIN><<<(A.batch + 16 * MT - 1) / (16 * MT), FR_WARPS * 32, smem, s>>>(S, A);
+  k_rows<MT, TRAIN><<<(A.batch + 16 * MT - 1) / (16 * MT), FR_WARPS * 32, rows_smem<TRAIN>(S, MT), s>>>(S, A);
   return cudaGetLastError();
+}
+// let k_rows have its shared memory on the current device (the attribute is per device)
+bool allow_rows() {
+  const auto allow = [](auto* kernel) {
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ROWS_SMEM_MAX) == cudaSuccess;
+  };
+  if (allow(k_rows<1, false>) && allow(k_rows<2, false>) && allow(k_rows<1, true>) && allow(k_rows<2, true>)) return true;
+  cudaGetLastError();
+  return false;
 }
 template <bool TRAIN>
 int rows_mt(const NetShape& S, int batch) {
@@ -1132,7 +1137,8 @@ lbm_status lbm_mlp_create(int n_in, int width, int depth, int n_pos, int n_cls, 
     S.nbias += m->fan_out[l];
     if (l > 0) toff += (long long)width * (l == L - 1 ? S.kp : width);
   }
-  m->fused = width % 64 == 0 && width <= 256 && n_in <= 64 && m->n_out <= 256 && rows_smem<true>(S, 1) <= ROWS_SMEM_MAX;
+  m->fused = width % 64 == 0 && width <= 256 && n_in <= 64 && m->n_out <= 256 &&
+             rows_smem<true>(S, 1) <= ROWS_SMEM_MAX && allow_rows();
   size_t max_part = 0;
   for (int l = 0; l < L; ++l) {
     const size_t s = (size_t)((max_batch + KSPLIT - 1) / KSPLIT) * m->fan_in[l] * m->fan_out[l];
