@@ -51,14 +51,16 @@ struct GemmArgs {
   long long ldz;
 };
 
-// 1 / (1 + exp(-z)).  The reciprocal by the hardware estimate and one Newton step (within 1 ulp): the
-// compiler's division carries a branch for subnormal quotients, which kept the 32 evaluations
-// of a thread's tile from overlapping (they were most of k_rows)
+// 1 / (1 + exp(-z)).  The reciprocal by the hardware estimate and one Newton step, of a quarter of the
+// denominator (rounded as the whole), so that the estimate of no finite one is subnormal.  Compared with the
+// rounded division for every float exp(-z) >= 0: the same bits wherever the quotient is normal (z > -87.3), within
+// 2^-149 below.  The evaluations are most of k_rows: 29 us for a batch of 4096, 31.5 us with a division.
 __device__ __forceinline__ float sigmoid_(float z) {
-  const float d = 1.0f + fminf(expf(-z), 1e38f);
+  const float e = expf(-z), d = fmaf(0.25f, e, 0.25f);
   float r;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(d));
-  return fmaf(r, fmaf(-d, r, 1.0f), r);
+  r = fmaf(r, fmaf(-d, r, 1.0f), r);
+  return e > 3.402823466e38f ? 0.0f : 0.25f * r;
 }
 // derivative of z s, s = sigmoid_(z)
 __device__ __forceinline__ float silu_slope(float z, float s) { return s * (1.0f + z * (1.0f - s)); }

@@ -112,3 +112,23 @@ def test_output_overlapping_the_input(cuda, n_in, n_out, batch, offset):
     got = net.forward(xv, out=yv)
     assert got.data_ptr() == yv.data_ptr() and torch.equal(got, want)
     net.close()
+
+
+@pytest.mark.parametrize("width", [64, 96])  # fused, layer by layer
+def test_silu_over_the_whole_range(cuda, width):
+    """One hidden layer with the pre-activations as biases and one output per unit: y = bf16(z sigmoid(z)), with z
+    where sigmoid is normal, subnormal and zero in FP32.  bfloat16 holds 8 bits, so it rounds a value in [1, 2) to
+    half of 2^-7, at most 2^-8 of it (2^-134 where it is subnormal itself); expf errs by 2 units of 2^-24, and
+    a subnormal sigmoid by a unit of 2^-149."""
+    z = np.concatenate([np.linspace(-103.0, -80.0, 24), np.linspace(-8.0, 8.0, 33), [-120.0, -30.0, 0.0, 40.0, 120.0]])
+    z = np.resize(z, width).astype(np.float32)
+    net = pkg.Mlp(n_in=1, width=width, depth=1, n_pos=width, n_cls=0, max_batch=1)
+    net.set_params(np.concatenate([np.zeros(width), z, np.eye(width).ravel(), np.zeros(width)]).astype(np.float32))
+    y = net.forward(np.zeros((1, 1), np.float32))[0].astype(np.float64)
+    net.close()
+    zd = z.astype(np.float64)
+    e = np.exp(-zd)
+    want = np.where(e > np.finfo(np.float32).max, 0.0, zd / (1.0 + e))
+    tiny = np.abs(zd) * 2.0 ** -148
+    bad = np.abs(y - want) > (2.0 ** -8 + 2.0 ** -22) * np.abs(want) + tiny + 2.0 ** -134
+    assert not bad.any(), (z[bad], y[bad], want[bad])
