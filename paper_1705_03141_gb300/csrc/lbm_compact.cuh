@@ -793,14 +793,14 @@ __global__ void k_init_c(CompactStore<BF16> st, Geom G, const __grid_constant__ 
   const int64_t sn = snode(G, x, y, z);
   const bool top = on_top(G, z);
   float* const tp = G.ctop + top_column(G, x, y);
-  equilibrium_pairs<DF>(r, b, u ? u[n] : 0.0, u ? u[N + n] : 0.0, u ? u[2 * N + n] : 0.0, K.alpha_r_d,
-                        [&](int t, DF fr, DF fb) {
-                          st.store(sn, t, speed2_of(t), K, narrow_(add_(fr, fb)));
-                          if (top) {
-                            tp[t * 32] = narrow_(fr);
-                            tp[(32 + t) * 32] = narrow_(fb);
-                          }
-                        });
+  equilibria<float>(r, b, u ? u[n] : 0.0, u ? u[N + n] : 0.0, u ? u[2 * N + n] : 0.0, K.alpha_r_d,
+                    [&](int t, auto fr, auto fb) {
+                      st.store(sn, t, speed2_of(t), K, (float)narrow_(add_(fr, fb)));
+                      if (top) {
+                        tp[t * 32] = (float)narrow_(fr);
+                        tp[(32 + t) * 32] = (float)narrow_(fb);
+                      }
+                    });
   dens[n] = make_float2((float)(r + b), (float)((r - b) / (r + b)));
 }
 

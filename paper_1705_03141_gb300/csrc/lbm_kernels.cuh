@@ -2148,19 +2148,47 @@ __device__ __forceinline__ void equilibrium_pairs(double rd, double bd, double u
   pair(tensor_index(1, -1, -1), rw, bw, rv, bv, sub_(dxy, u2));
 }
 
+// the same direction by direction as the equation stands, whatever the values (an infinite density at rest
+// gives infinite populations; in opposite pairs it would meet a zero factor)
+template <class Put>
+__device__ __forceinline__ void equilibrium_each(double r, double b, double u0, double u1, double u2, double ar,
+                                                 const Put& put) {
+  const double uu = u0 * u0 + u1 * u1 + u2 * u2;
+#pragma unroll
+  for (int t = 0; t < 27; ++t) {
+    const double w = weight_of(t), cu = cx_of(t) * u0 + cy_of(t) * u1 + cz_of(t) * u2;
+    const double poly = w * (3.0 * cu + 4.5 * cu * cu - 1.5 * uu);
+    const double vr = t == REST ? ar : 27.0 / 19.0 * (1.0 - ar) * w, vb = t == REST ? 8.0 / 27.0 : w;
+    put(t, r * (vr + poly), b * (vb + poly));
+  }
+}
+// Opposite pairs where their terms neither overflow nor, for pairs of FP32 values, lose a tail.
+template <typename R>
+__device__ __forceinline__ bool pairs_hold(double rho) {
+  const float h = fabsf((float)rho);
+  return h <= 1e15f && (std::is_same<R, double>::value || h >= 1e-30f || rho == 0.0);
+}
+template <typename R, class Put>
+__device__ __forceinline__ void equilibria(double r, double b, double u0, double u1, double u2, double ar,
+                                           const Put& put) {
+  const bool hold = pairs_hold<R>(r) && pairs_hold<R>(b) && fabsf((float)u0) <= 1e4f && fabsf((float)u1) <= 1e4f &&
+                    fabsf((float)u2) <= 1e4f;
+  if (hold) equilibrium_pairs<typename WideOf<R>::type>(r, b, u0, u1, u2, ar, put);
+  else equilibrium_each(r, b, u0, u1, u2, ar, put);
+}
+
 // f^k = f^{k(e)}(rho_k, u, alpha_k), Phi = 0; written in layout 0.
 template <class Store>
 __global__ void k_init(Store st, Geom G, const __grid_constant__ KConst<typename DensOf<Store>::real> K,
                        const double* __restrict__ rr, const double* __restrict__ rb, const double* __restrict__ u) {
   using R = typename DensOf<Store>::real;
-  using T = typename WideOf<R>::type;
   const int64_t N = (int64_t)G.nx * G.ny * G.nz;
   const int64_t n = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (n >= N) return;
   const int x = (int)(n % G.nx), y = (int)((n / G.nx) % G.ny), z = (int)(n / ((int64_t)G.nx * G.ny));
   const int64_t sn = snode(G, x, y, z);
-  equilibrium_pairs<T>(rr[n], rb[n], u ? u[n] : 0.0, u ? u[N + n] : 0.0, u ? u[2 * N + n] : 0.0, K.alpha_r_d,
-                       [&](int t, T fr, T fb) { store_pair(st, K, sn, t, (R)narrow_(fr), (R)narrow_(fb)); });
+  equilibria<R>(rr[n], rb[n], u ? u[n] : 0.0, u ? u[N + n] : 0.0, u ? u[2 * N + n] : 0.0, K.alpha_r_d,
+                [&](int t, auto fr, auto fb) { store_pair(st, K, sn, t, (R)narrow_(fr), (R)narrow_(fb)); });
 }
 
 // one direction (paper order pdir) of the canonical [2][27][N] FP64 array <-> storage

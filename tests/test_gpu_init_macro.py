@@ -56,3 +56,33 @@ def test_initial_populations_and_macroscopic_sums(shape, storage, eps_f, eps_m):
         mom = sum(int(c[i][a]) * (g[0, i] + g[1, i]) for i in range(27))
         F = (rho - np.longdouble(real(p["rho_b0"]))) * np.longdouble(real(p["g"][a]))
         assert np.all(np.abs(v[a] - (mom + F / 2) / rho) <= 4 * eps_m)
+
+
+@pytest.mark.parametrize("storage", ["f64", "f32"])
+def test_initial_fields_out_of_the_pairs_range(storage):
+    """Infinities, densities that FP32 cannot hold or whose tails it loses, and large velocities: the populations are
+    the FP64 equilibria, rounded once to the storage."""
+    shape = (33, 5, 4)
+    w = _work(shape)
+    rr, rb, u = L.initial_fields(w, seed=5, u_amp=0.1)
+    n = [(0, 0, 0), (0, 1, 5), (1, 2, 32), (2, 3, 31), (3, 4, 7), (2, 0, 0), (1, 1, 1), (3, 0, 20), (1, 3, 3)]
+    rr[n[0]], rr[n[1]], rb[n[2]], rr[n[3]] = np.inf, 1e39, 4e38, 1e-36
+    rb[n[4]], rr[n[4]], u[(1,) + n[5]], u[(2,) + n[6]] = 2e-38, 1e-44, 1e20, np.inf
+    rr[n[7]], rb[n[7]], rb[n[8]] = 0.0, 1e-42, np.nan
+    u[(slice(None),) + n[0]] = 0.0
+    lat = pkg.Lattice(shape, w["params"], storage=storage)
+    lat.init_fields(rr, rb, u)
+    orc = oracle.Oracle(shape, w["params"])
+    orc.init_fields(rr, rb, u)
+    with np.errstate(all="ignore"):
+        ref = orc.f.reshape((2, 27) + shape[::-1])
+        ref = ref if storage == "f64" else ref.astype(np.float32).astype(np.float64)
+        f = lat.get_populations().reshape(ref.shape)
+        for at in n:
+            a, b = f[(slice(None), slice(None)) + at], ref[(slice(None), slice(None)) + at]
+            assert np.array_equal(np.isnan(a), np.isnan(b)) and np.array_equal(np.isinf(a), np.isinf(b)), at
+            ok = np.isfinite(b)
+            # FP64 operations in another order, and for FP32 storage the unit by which they may round differently
+            eps = 2.0 ** -48 if storage == "f64" else 2.0 ** -23
+            assert np.all(np.abs(a[ok] - b[ok]) <= eps * np.abs(b[ok]) + (storage == "f32") * 2.0 ** -149), at
+    lat.close()
