@@ -806,28 +806,34 @@ __global__ void k_init_c(CompactStore<BF16> st, Geom G, const __grid_constant__ 
 
 // rho_r, rho_b, u (Eq. Momentum) into FP64 device buffers (any may be null); rho_r from the
 // (rho, phi) field of pass 1 for the current state
-// (128x128x512: 1360 us with every node on the general map and the outflow plane's test in the loop, 600 now)
+// (128x128x512: 1360 us with every node on the general map and the outflow plane's test in the loop, 616 now, 592
+// with sums in FP32 pairs)
 template <bool BF16>
-__global__ void k_macro_c(CompactStore<BF16> st, Geom G, const __grid_constant__ KConst<float> K, int layout,
-                          const float2* __restrict__ dens, double* __restrict__ rr, double* __restrict__ rb,
-                          double* __restrict__ u) {
+__global__ void __launch_bounds__(256, 4)
+    k_macro_c(CompactStore<BF16> st, const __grid_constant__ Geom G, const __grid_constant__ KConst<float> K, int layout,
+              const float2* __restrict__ dens, double* __restrict__ rr, double* __restrict__ rb,
+              double* __restrict__ u) {
   const int64_t N = (int64_t)G.nx * G.ny * G.nz;
   const int64_t n = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (n >= N) return;
   const int x = (int)(n % G.nx), y = (int)((n / G.nx) % G.ny), z = (int)(n / ((int64_t)G.nx * G.ny));
   const bool top = on_top(G, z);
-  DF srho = {0.f, 0.f}, sred = {0.f, 0.f}, m[3] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
+  TF srho{}, sred{}, m[3] = {TF{}, TF{}, TF{}};
   float f[27];
+  const auto momentum = [&m](int t, TF s) {
+    if (cx_of(t)) acc_(m[0], cx_of(t) > 0 ? s : neg_(s));
+    if (cy_of(t)) acc_(m[1], cy_of(t) > 0 ? s : neg_(s));
+    if (cz_of(t)) acc_(m[2], cz_of(t) > 0 ? s : neg_(s));
+  };
+  const float* const tp = top ? G.ctop + top_column(G, x, y) : nullptr;
   if (top) {
-    const float* tp = G.ctop + top_column(G, x, y);
 #pragma unroll
     for (int t = 0; t < 27; ++t) {
-      const DF s = two_sum(tp[t * 32], tp[(32 + t) * 32]);
+      TF s;
+      sum2_(s, tp[t * 32], tp[(32 + t) * 32]);
       acc_(sred, tp[t * 32]);
       acc_(srho, s);
-      if (cx_of(t)) acc_(m[0], cx_of(t) > 0 ? s : neg_(s));
-      if (cy_of(t)) acc_(m[1], cy_of(t) > 0 ? s : neg_(s));
-      if (cz_of(t)) acc_(m[2], cz_of(t) > 0 ? s : neg_(s));
+      momentum(t, s);
     }
   } else {
     if (fast_row(G, y, z)) {
@@ -846,26 +852,39 @@ __global__ void k_macro_c(CompactStore<BF16> st, Geom G, const __grid_constant__
         f[t] = st.load(node, dir, speed2_of(t), K);
       }
     }
+    sum2_(srho, f[0], f[1]);
 #pragma unroll
-    for (int t = 0; t < 27; ++t) acc_(srho, f[t]);
+    for (int t = 2; t < 27; ++t) acc_(srho, f[t]);
   }
   if (!top && u) {
 #pragma unroll
     for (int t = 14; t < 27; ++t) {
-      const DF d = two_sum(f[t], -f[26 - t]);
-      if (cx_of(t)) acc_(m[0], cx_of(t) > 0 ? d : neg_(d));
-      if (cy_of(t)) acc_(m[1], cy_of(t) > 0 ? d : neg_(d));
-      if (cz_of(t)) acc_(m[2], cz_of(t) > 0 ? d : neg_(d));
+      TF d;
+      sum2_(d, f[t], -f[26 - t]);
+      momentum(t, d);
     }
   }
-  if (rr || rb) {
-    const double rho = to_f64(srho);
-    double red = to_f64(sred);
-    if (!top) red = 0.5 * rho * (1.0 + (double)dens[n].y);
-    if (rr) rr[n] = red;
-    if (rb) rb[n] = rho - red;
+  double rho = to_f64(srho), red = top ? to_f64(sred) : 0.0, j[3];
+  if (u) {
+#pragma unroll
+    for (int a = 0; a < 3; ++a) j[a] = to_f64(m[a]);
   }
-  if (u) write_velocity(K, srho, m, u, n, N);
+  if (!(whole_(srho) && whole_(sred) && whole_(m[0]) && whole_(m[1]) && whole_(m[2]))) {  // infinities stay infinite
+    rho = red = j[0] = j[1] = j[2] = 0.0;
+#pragma unroll
+    for (int t = 0; t < 27; ++t) {
+      const double s = top ? (double)tp[t * 32] + (double)tp[(32 + t) * 32] : (double)f[t];
+      if (top) red += (double)tp[t * 32];
+      rho += s;
+      j[0] += cx_of(t) * s;
+      j[1] += cy_of(t) * s;
+      j[2] += cz_of(t) * s;
+    }
+  }
+  if (!top) red = 0.5 * rho * (1.0 + (double)dens[n].y);
+  if (rr) rr[n] = red;
+  if (rb) rb[n] = rho - red;
+  if (u) write_velocity(K, rho, j, u, n, N);
 }
 
 // one direction (paper order) of the canonical FP64 arrays <- storage, colours rebuilt

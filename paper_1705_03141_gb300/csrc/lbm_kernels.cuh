@@ -2250,23 +2250,67 @@ __global__ void k_top_from_state(Store st, Geom G, const __grid_constant__ KCons
   }
 }
 
-// u = (j + F/2) / rho (Eq. Momentum) of node n into the three components of u
-template <typename T, typename R>
-__device__ __forceinline__ void write_velocity(const KConst<R>& K, T rho, const T j[3], double* __restrict__ u,
-                                               int64_t n, int64_t N) {
-  T k = wide_<T>(0.0);
-  if (K.force_mode == FORCE_BUOYANCY || K.force_mode == FORCE_DISPERSED) k = sub_(rho, wide_<T>((double)K.rho_ref));
-  else if (K.force_mode == FORCE_UNIFORM) k = wide_<T>(1.0);
+// u = (j + F/2) / rho (Eq. Momentum) of node n into the three components of u.  FP32-arithmetic storages
+// share one reciprocal (the FP32 estimate, one Newton step: 46 bits) and correct each quotient by its
+// remainder, which rounds it within 2^-40 of correctly; an FP64 division is about three times the
+// instructions on the FP64 pipe.
+template <typename R>
+__device__ __forceinline__ void write_velocity(const KConst<R>& K, double rho, const double j[3],
+                                               double* __restrict__ u, int64_t n, int64_t N) {
+  double k = 0.0;
+  if (K.force_mode == FORCE_BUOYANCY || K.force_mode == FORCE_DISPERSED) k = rho - (double)K.rho_ref;
+  else if (K.force_mode == FORCE_UNIFORM) k = 1.0;
+  const float rf = (float)rho;
+  const bool quick = std::is_same<R, float>::value && rf > 1e-30f && rf < 1e30f;
+  double x = 0.0;
+  if (quick) {
+    x = wide_bits(__frcp_rn(rf));
+    x = fma(x, fma(-rho, x, 1.0), x);
+  }
 #pragma unroll
-  for (int a = 0; a < 3; ++a)
-    u[a * N + n] = to_f64(div_(mad_(k, wide_<T>(0.5 * (double)K.g[a]), j[a]), rho));
+  for (int a = 0; a < 3; ++a) {
+    const double v = fma(k, 0.5 * (double)K.g[a], j[a]);
+    if (quick) {
+      const double q = v * x;
+      u[a * N + n] = fma(fma(-q, rho, v), x, q);
+    } else {
+      u[a * N + n] = v / rho;
+    }
+  }
 }
 
-// rho_r, rho_b, u (Eq. Momentum) into FP64 device buffers (any may be null); on the 128x128x512 jet f16
-// 692 -> 567 us, FP32 632 -> 567 against the general map on every node
+// densities and momentum of a node in FP64, population after population: where the lossless sums do not
+// hold (infinities, NaN, overflow of FP32)
+template <class Store, typename R>
+__device__ __noinline__ void macro_plain(const Store& st, const Geom& G, const KConst<R>& K, int layout, int x, int y,
+                                         int z, double& r, double& b, double j[3]) {
+  NodeMap nm;
+  nm.init(G, x, y, z);
+  r = b = j[0] = j[1] = j[2] = 0.0;
+#pragma unroll 1
+  for (int t = 0; t < 27; ++t) {
+    int64_t node;
+    int dir;
+    slot_of(nm, layout, t, node, dir);
+    R fr, fb;
+    st.load_rb(node, dir, speed2_of(t), K, fr, fb);
+    r += (double)fr;
+    b += (double)fb;
+    const double s = (double)fr + (double)fb;
+    j[0] += cx_of(t) * s;
+    j[1] += cy_of(t) * s;
+    j[2] += cz_of(t) * s;
+  }
+}
+
+// rho_r, rho_b, u (Eq. Momentum) into FP64 device buffers (any may be null).  FP32-arithmetic storages sum
+// without loss (TF); FP64 additions alone would take about 3 ms for the 128x128x512 jet, which takes 641 us
+// (FP32) and 655 us (packed half) like this and 557 with sums in FP32 pairs, 2^-48 off.  Three blocks per SM
+// (80 registers): 1060 us with two.
 template <class Store>
-__global__ void k_macro(Store st, Geom G, const __grid_constant__ KConst<typename DensOf<Store>::real> K, int layout,
-                        double* __restrict__ rr, double* __restrict__ rb, double* __restrict__ u) {
+__global__ void __launch_bounds__(256, std::is_same<typename DensOf<Store>::real, float>::value ? 3 : 1)
+    k_macro(Store st, const __grid_constant__ Geom G, const __grid_constant__ KConst<typename DensOf<Store>::real> K,
+            int layout, double* __restrict__ rr, double* __restrict__ rb, double* __restrict__ u) {
   using R = typename DensOf<Store>::real;
   const int64_t N = (int64_t)G.nx * G.ny * G.nz;
   const int64_t n = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -2297,23 +2341,26 @@ __global__ void k_macro(Store st, Geom G, const __grid_constant__ KConst<typenam
       st.load_rb(node, dir, speed2_of(t), K, fr[t], fb[t]);
     }
   }
-  using T = typename WideOf<R>::type;
-  T sr = wide_<T>(0.0), sb = wide_<T>(0.0);
-#pragma unroll
-  for (int t = 0; t < 27; ++t) {
+  using T = typename SumOf<R>::type;
+  T sr, sb, m[3] = {T{}, T{}, T{}};
+  sum2_(sr, fr[REST], fr[0]);
+  sum2_(sb, fb[REST], fb[0]);
+  // pair after pair, so that a pair's registers are free after it
+  const auto pair = [&](int t) {
     acc_(sr, fr[t]);
     acc_(sb, fb[t]);
-  }
-  if (rr) rr[n] = to_f64(sr);
-  if (rb) rb[n] = to_f64(sb);
+    if (t != 26) {
+      acc_(sr, fr[26 - t]);
+      acc_(sb, fb[26 - t]);
+    }
+  };
   if (u) {
-    // momentum from the 13 differences of opposite populations
-    T m[3] = {wide_<T>(0.0), wide_<T>(0.0), wide_<T>(0.0)};
 #pragma unroll
-    for (int t = 14; t < 27; ++t) {
-      T d = wide_<T>(0.0);
-      acc_(d, fr[t]);
-      acc_(d, -fr[26 - t]);
+    for (int t = 26; t > REST; --t) {
+      pair(t);
+      // momentum from the 13 differences of opposite populations
+      T d;
+      sum2_(d, fr[t], -fr[26 - t]);
       acc_(d, fb[t]);
       acc_(d, -fb[26 - t]);
       const int c[3] = {cx_of(t), cy_of(t), cz_of(t)};
@@ -2323,8 +2370,24 @@ __global__ void k_macro(Store st, Geom G, const __grid_constant__ KConst<typenam
         if (c[a] < 0) acc_(m[a], neg_(d));
       }
     }
-    write_velocity(K, add_(sr, sb), m, u, n, N);
+  } else {
+#pragma unroll
+    for (int t = 26; t > REST; --t) pair(t);
   }
+  double r, b, j[3];
+  if (whole_(sr) && whole_(sb) && whole_(m[0]) && whole_(m[1]) && whole_(m[2])) {
+    r = to_f64(sr);
+    b = to_f64(sb);
+    if (u) {
+#pragma unroll
+      for (int a = 0; a < 3; ++a) j[a] = to_f64(m[a]);
+    }
+  } else {
+    macro_plain(st, G, K, layout, x, y, z, r, b, j);
+  }
+  if (rr) rr[n] = r;
+  if (rb) rb[n] = b;
+  if (u) write_velocity(K, r + b, j, u, n, N);
 }
 
 // ---------------------------------------------------------------------------

@@ -1,11 +1,12 @@
-"""Initial populations and macroscopic fields: FP32-arithmetic storages take FP64 fields in and out
-through head + tail FP32 pairs.
+"""Initial populations and macroscopic fields: FP32-arithmetic storages take FP64 fields in through head + tail
+FP32 pairs and out through lossless sums of FP32 values.
 
 Bounds.  A pair holds 48 bits and each operation on pairs errs by a few units of 2^-47 of its
 operands, so an initial FP32 population is the FP64 value (a sum of terms at most 8 times its size
-for |u| <= 0.15) rounded once: 2^-24 of it, plus 2^-40.  A macroscopic density, a sum of 27 stored
-values, errs by less than 27 * 2^-46 < 2^-41 of it; the velocity, from 54 values and one quotient,
-by less than 2^-40 of the largest possible speed 1.  FP64 storage: 2^-48 for all.
+for |u| <= 0.15) rounded once: 2^-24 of it, plus 2^-40.  A macroscopic density is the sum of 27 stored
+values rounded to FP64 in two additions, 2^-52 of it; the velocity, of a speed below 1, carries the roundings of
+its momentum (2), of rho (3 in the quotient and the force), of the force and of the quotient: 8 units of 2^-53.
+FP64 storage sums in FP64, at most 27 roundings of a partial sum: 2^-48 for all.
 """
 import numpy as np
 import pytest
@@ -27,8 +28,8 @@ def _work(shape):
 
 
 @pytest.mark.parametrize("shape", SHAPES)
-@pytest.mark.parametrize("storage,eps_f,eps_m", [("f64", 2.0 ** -48, 2.0 ** -48), ("f32", 2.0 ** -24 + 2.0 ** -40, 2.0 ** -40),
-                                                 ("f16", None, 2.0 ** -40), ("bf16", None, 2.0 ** -40)])
+@pytest.mark.parametrize("storage,eps_f,eps_m", [("f64", 2.0 ** -48, 2.0 ** -48), ("f32", 2.0 ** -24 + 2.0 ** -40, 2.0 ** -52),
+                                                 ("f16", None, 2.0 ** -52), ("bf16", None, 2.0 ** -52)])
 def test_initial_populations_and_macroscopic_sums(shape, storage, eps_f, eps_m):
     w = _work(shape)
     rr, rb, u = L.initial_fields(w, seed=5, u_amp=0.1)
@@ -86,3 +87,30 @@ def test_initial_fields_out_of_the_pairs_range(storage):
             eps = 2.0 ** -48 if storage == "f64" else 2.0 ** -23
             assert np.all(np.abs(a[ok] - b[ok]) <= eps * np.abs(b[ok]) + (storage == "f32") * 2.0 ** -149), at
     lat.close()
+
+
+@pytest.mark.parametrize("storage", ["f64", "f32"])
+def test_macroscopic_fields_of_infinite_populations(storage):
+    """A node with an infinite, an overflowing, a NaN population: as the sums in FP64 have it, other nodes untouched."""
+    shape = (33, 5, 4)
+    w = _work(shape)
+    rr, rb, u = L.initial_fields(w, seed=5, u_amp=0.1)
+    lat = pkg.Lattice(shape, w["params"], storage=storage)
+    lat.init_fields(rr, rb, u)
+    f = lat.get_populations().reshape((2, 27) + shape[::-1])
+    clean = lat.macro()
+    f[0, 3, 1, 2, 4] = np.inf
+    f[:, 5:7, 2, 3, 32] = 3e38  # the density of each colour is beyond FP32
+    f[1, 9, 3, 0, 7] = np.nan
+    lat.set_populations(f)
+    r, b, v = lat.macro()
+    lat.close()
+    assert r[1, 2, 4] == np.inf and b[1, 2, 4] == clean[1][1, 2, 4]
+    assert np.isnan(b[3, 0, 7]) and r[3, 0, 7] == clean[0][3, 0, 7] and np.all(np.isnan(v[:, 3, 0, 7]))
+    for a, k in ((r, 0), (b, 1)):
+        want = f[k, :, 2, 3, 32].astype(np.float32).astype(np.longdouble).sum() if storage == "f32" else f[k, :, 2, 3, 32].sum()
+        assert abs(a[2, 3, 32] - want) <= 2.0 ** -48 * want
+    hit = np.zeros(r.shape, bool)
+    hit[1, 2, 4] = hit[2, 3, 32] = hit[3, 0, 7] = True
+    for a, c in zip((r, b, *v), (clean[0], clean[1], *clean[2])):
+        assert np.array_equal(a[~hit], c[~hit])
