@@ -429,6 +429,7 @@ lbm_status lbm_create(int nx, int ny, int nz, const lbm_params* p, lbm** out) {
   h->shape = p->block != 0 ? p->block - 1 : (h->variant == 3 && p->storage == LBM_STORE_F32 ? 1 : 0);
   // compact storage: the TMA-pipelined pass 1 wherever it applies (522 against 711 us a step on the jet)
   if (h->ks->compact && p->block == 0 && pipelined_ok(nx, ny, nz, p)) h->shape = 3;
+  if (p->storage == LBM_STORE_F64) h->shape = 0;  // node after node, whatever was asked for
 
   Geom& G = h->G;
   G.nx = nx;

@@ -679,7 +679,7 @@ __global__ void __launch_bounds__(NTHREADS, 4)
 
   float gphi[3], grho[3];
   const int lx = threadIdx.x + 1, ly = threadIdx.y + 1, lz = threadIdx.z + 1;
-  tile_gradients<float>(tile, lx, ly, lz, gphi, grho);
+  tile_gradients(tile, lx, ly, lz, gphi, grho);
   float f[27];
   float4 record;
   if (is_inlet(G, x, y, z)) {

@@ -910,20 +910,16 @@ __device__ __forceinline__ void pair_gradients(const Get& get, V g[3]) {
   g[2] = O::fma(w1, O::sub(get(0, 0, 1), get(0, 0, -1)), g[2]);
 }
 
-template <typename R, typename DT, int TXv = TX, int TYv = TY>
-__device__ __forceinline__ void tile_gradients(const DT* tile, int lx, int ly, int lz, R gphi[3], R grho[3]) {
-  const DT* const c = tile + lx + TXv * (ly + TYv * lz);
-  if constexpr (std::is_same<R, float>::value && std::is_same<DT, float2>::value) {
-    float2 g[3];
-    pair_gradients<float2>([c](int x, int y, int z) { return c[x + TXv * (y + TYv * z)]; }, g);
+template <int TXv = TX, int TYv = TY>
+__device__ __forceinline__ void tile_gradients(const float2* tile, int lx, int ly, int lz, float gphi[3],
+                                               float grho[3]) {
+  const float2* const c = tile + lx + TXv * (ly + TYv * lz);
+  float2 g[3];
+  pair_gradients<float2>([c](int x, int y, int z) { return c[x + TXv * (y + TYv * z)]; }, g);
 #pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      grho[k] = g[k].x;
-      gphi[k] = g[k].y;
-    }
-  } else {
-    pair_gradients<R>([c](int x, int y, int z) { return (R)c[x + TXv * (y + TYv * z)].x; }, grho);
-    pair_gradients<R>([c](int x, int y, int z) { return (R)c[x + TXv * (y + TYv * z)].y; }, gphi);
+  for (int k = 0; k < 3; ++k) {
+    grho[k] = g[k].x;
+    gphi[k] = g[k].y;
   }
 }
 
@@ -1307,7 +1303,7 @@ __global__ void __launch_bounds__(B::NT, MINB)
                      const typename DensOf<Store>::type* __restrict__ dens, long long* __restrict__ counter,
                      const FusedIO io, const __grid_constant__ CUtensorMap dmap, int tma, const TileSplit bt,
                      int bmode) {
-  using R = typename DensOf<Store>::real;  // compute type: FP64 for FP64 storage, FP32 otherwise
+  using R = typename DensOf<Store>::real;  // FP32: FP64 storage runs k_collide_stream_lin
   using DT = typename DensOf<Store>::type;
   __shared__ __align__(128) DT tile[B::TILET];
   __shared__ float2 prow[FUSED ? B::NW * 9 * B::TX : 1];
@@ -1338,7 +1334,7 @@ __global__ void __launch_bounds__(B::NT, MINB)
 
   // block-uniform: the tile comes by TMA (no periodic face crossed)
   bool via_tma = false;
-  if constexpr (!FUSED && std::is_same<DT, float2>::value) {
+  if constexpr (!FUSED) {
     via_tma = tma != 0 && !tile_wraps<B>(G, x0, y0, z0);
     if (via_tma) {
       if (tid == 0) {
@@ -1433,7 +1429,7 @@ __global__ void __launch_bounds__(B::NT, MINB)
 
   if (active) {
     R gphi[3], grho[3];
-    tile_gradients<R, DT, B::TXT, B::TY>(tile, threadIdx.x + 2, threadIdx.y + 1, threadIdx.z + 1, gphi, grho);
+    tile_gradients<B::TXT, B::TY>(tile, threadIdx.x + 2, threadIdx.y + 1, threadIdx.z + 1, gphi, grho);
 
     R f[27];
     Recol<R> rc;
@@ -1765,7 +1761,7 @@ __global__ void __launch_bounds__(NTHREADS, MINB)
         rho_r += fr;
       }
       float gphi[3], grho[3];
-      tile_gradients<float>(ts, threadIdx.x + 1, threadIdx.y + 1, threadIdx.z + 1, gphi, grho);
+      tile_gradients(ts, threadIdx.x + 1, threadIdx.y + 1, threadIdx.z + 1, gphi, grho);
       float f[27];
       Recol<float> rc;
       if (is_inlet(G, x, y, z)) {

@@ -25,7 +25,6 @@ struct StoreTraits;
 template <>
 struct StoreTraits<PlainStore<double>> {
   static constexpr bool paired = false;
-  static constexpr int minb = 1, minb2 = 1, minb_pf = 1;
   static PlainStore<double> make(void* p, const Geom& G) { return {static_cast<double*>(p), G.Ns}; }
 };
 template <>
@@ -96,7 +95,7 @@ struct Launch {
   // the tiles are then loaded as for boxes that cross a periodic face, with the same values.
   template <class B>
   static bool dens_map(const Geom& G, const void* dens, CUtensorMap* m) {
-    if (!std::is_same<DT, float2>::value || (G.nx & 1) || getenv("LBM_NO_TMA") != nullptr) return false;
+    if ((G.nx & 1) || getenv("LBM_NO_TMA") != nullptr) return false;
     const EncodeTiledFn enc = encode_tiled();
     if (!enc) return false;
     char* base = const_cast<char*>(static_cast<const char*>(dens)) - (size_t)G.nx * G.ny * sizeof(DT);

@@ -160,7 +160,7 @@ __global__ void __launch_bounds__(TP_THREADS, TP_MINB)
     const bool act = x < G.nx;
     float rho_r = 0.f, ft[27], gphi[3], grho[3];
     if (act) {
-      tile_gradients<float, float2, B::TXT, B::TY>(dt, lane + 2, ty + 1, tz + 1, gphi, grho);
+      tile_gradients<B::TXT, B::TY>(dt, lane + 2, ty + 1, tz + 1, gphi, grho);
       float acc = 0.f;
       if (!ODD) {
         const unsigned char* const b0 = stg + row * TP_ROW + lane * 4;

@@ -55,3 +55,10 @@ def test_fp64_rounding_no_larger_than_moment_by_moment(cuda):
         lat.close()
     _, blue, u = np.mean(err, axis=0)
     assert blue < 3.57e-16 and u < 7.24e-14
+
+
+@pytest.mark.parametrize("block", [0, 1, 2, 3])
+def test_fp64_reports_block_one(cuda, block):
+    lat = pkg.Lattice((8, 8, 8), L.static_droplet(n=8, R=2.0)["params"], storage="f64", block=block)
+    assert lat.block == 1
+    lat.close()
