@@ -47,3 +47,37 @@ def test_face_rows_match_the_oracle(cuda, shape, storage, variant):
                 err = np.max(np.abs(g - orc.f))
                 assert err < tol, (bx, by, z, n, err, tol)
             lat.close()
+
+
+# more than two tiles along y and z, a ragged last block and none: the pipelined compact density pass, whose face
+# rows read the colour records from global memory (x faces reflect; every pair of y and z faces)
+@pytest.mark.parametrize("storage", ["c16", "cbf16"])
+@pytest.mark.parametrize("shape", [(32, 9, 6), (45, 14, 7)])
+def test_pipelined_compact_face_rows(cuda, shape, storage):
+    """Bitwise the one-block pass, and (half) within its budget of the oracle."""
+    for by in (0, 1, 2):
+        for z in Z + [(1, 1)]:
+            p = dict(L.parity_cases()[3 if z[0] == 3 else 1][1]["params"])
+            p["bc"] = (2, 2, by, by) + z
+            if z[0] == 3:
+                p["inflow"] = dict(p["inflow"], xc=0.5 * (shape[0] - 1), yc=0.5 * (shape[1] - 1), D=2.0)
+            w = dict(name="faces", shape=shape, params=p, fields=("random_blobs", dict(seed=3, blobs=2)), steps=4)
+            rr, rb, u = L.initial_fields(w, seed=4, u_amp=0.02)
+            lats = [pkg.Lattice(shape, p, storage=storage, block=b) for b in (1, 4)]
+            assert [lat.block for lat in lats] == [1, 4]
+            for lat in lats:
+                lat.init_fields(rr, rb, u)
+            orc = oracle.Oracle(shape, p)
+            orc.init_fields(rr, rb, u)
+            for n in (1, 2, 3, 4):
+                for lat in lats:
+                    lat.step(1)
+                orc.step(1)
+                a, b = (lat.get_populations() for lat in lats)
+                assert np.array_equal(a, b), (by, z, n)
+                for x, y in zip(*(lat.macro() for lat in lats)):
+                    assert np.array_equal(x, y), (by, z, n)
+                if storage == "c16":
+                    assert np.max(np.abs(b - orc.f)) < 2e-3 * np.max(orc.f), (by, z, n)
+            for lat in lats:
+                lat.close()
