@@ -137,6 +137,9 @@ const char* validate(int nx, int ny, int nz, const lbm_params* p) {
   // (up to 54 values per node) must hold fewer than 2^31 elements
   if ((double)align_up((size_t)nx, 32) * ny * 54.0 >= 2147483647.0 - 65536.0)
     return "xy plane too large (nx rounded up to 32, times ny, times 54 must stay below 2^31)";
+  // and a wrap in z, by 32-bit node offsets of the padded rows
+  if (p->bc[4] == LBM_BC_PERIODIC && (double)align_up((size_t)nx, 32) * ny * nz >= 2147483647.0)
+    return "box too large for periodic z faces (nx rounded up to 32, times ny * nz must stay below 2^31)";
   if (!(p->rho_r0 > 0) || !(p->rho_b0 > 0)) return "rho_r0 and rho_b0 must be > 0";
   const double ab = 8.0 / 27.0, ar = 1.0 - (1.0 - ab) / (p->rho_r0 / p->rho_b0);
   if (!(ar >= 0.0 && ar < 1.0)) return "density ratio rho_r0/rho_b0 must be >= 19/27 (alpha_r in [0,1))";
@@ -438,6 +441,7 @@ lbm_status lbm_create(int nx, int ny, int nz, const lbm_params* p, lbm** out) {
   G.nz = nz;
   G.Ns = Ns;
   for (int f = 0; f < 6; ++f) G.bc[f] = p->bc[f];
+  G.rows = lbmk::row_shifts(G);
   G.inflow = 0;
   G.xc = G.yc = G.r2 = 0.0;
   G.ctop = nullptr;
@@ -887,6 +891,20 @@ lbm_status lbm_selfcheck(const char** msg) {
   if (fabs(sw - 1.0) > 1e-15 || fabs(s2 - 1.0 / 3.0) > 1e-15) {
     if (msg) *msg = "weights do not satisfy sum w = 1, sum w c_x^2 = 1/3";
     return LBM_EINVAL;
+  }
+  // rows wrap in z by 32-bit shifts only where every shift, with 54 values a node, fits
+  for (int k = 0; k < 2; ++k) {
+    Geom g;
+    memset(&g, 0, sizeof g);  // periodic faces
+    g.nx = 3;
+    g.nxs = 32;
+    g.ny = 6000;
+    g.nz = 6627 + k;
+    const int64_t sz = (int64_t)(g.nxs >> 5) * 54 * g.ny;
+    if (lbmk::row_shifts(g) != (k == 0) || (k == 0 && g.nz * sz >= (1ll << 31))) {
+      if (msg) *msg = "row shifts are used beyond 32 bits";
+      return LBM_EINVAL;
+    }
   }
   return LBM_OK;
 }

@@ -64,6 +64,7 @@ struct Geom {
   int nxs;        // storage row length: nx rounded up to a multiple of 32 (whole 32-node blocks per row)
   int64_t Ns;     // storage nodes: nxs*ny*(nz+2) rounded up (ghost planes z=-1, z=nz)
   int bc[6];
+  int rows;       // rows may stream by row shifts (row_shifts)
   int inflow;     // inlet disk active on z = 0
   double xc, yc, r2;
   float* ctop;    // compact storage with an outflow face: the top plane's populations per colour
@@ -256,7 +257,7 @@ struct NodeMap {
 struct AoRow {
   int64_t e[3];
   int dxm, dxp;        // e[0] - e[1] and e[2] - e[1]
-  int ym, yp, zm, zp;  // row shifts in units of 32 elements (below 2^31 up to 2.5e9 padded nodes)
+  int ym, yp, zm, zp;  // row shifts in units of 32 elements (below 2^31: row_shifts)
   // the node's storage block (x >> 5) + (nxs / 32)(y + ny (z + 1)) fits 32 bits; within a block the
   // x neighbours are one element away, across a block edge one block of PLANES planes minus 31.
   // INTERIOR: the row touches no y or z face
@@ -296,15 +297,21 @@ struct AoRow {
   }
 };
 
+// Where rows have row shifts at all (Geom::rows): no x face bounces back, and a wrap in z, which moves a row by
+// nearly the whole box, fits 32 bits with 54 values a node: 1.27e9 padded nodes (a box passes that within the
+// GPU's memory only in FP32 storage with rows of up to 8 nodes).
+inline bool row_shifts(const Geom& g) {
+  const bool fit = g.bc[4] != BC_PERIODIC || (int64_t)(g.nxs / 32) * 54 * g.ny * (g.nz + 1) < (1ll << 31);
+  return g.bc[0] != BC_NOSLIP && g.bc[1] != BC_NOSLIP && fit;
+}
 // rows whose streaming map is AoRow's
 __device__ __forceinline__ bool fast_row(const Geom& g, int y, int z) {
-  return g.bc[0] != BC_NOSLIP && g.bc[1] != BC_NOSLIP && (y > 0 || g.bc[2] != BC_NOSLIP) &&
-         (y < g.ny - 1 || g.bc[3] != BC_NOSLIP) && (z > 0 || g.bc[4] != BC_NOSLIP) &&
-         (z < g.nz - 1 || g.bc[5] != BC_NOSLIP);
+  return g.rows && (y > 0 || g.bc[2] != BC_NOSLIP) && (y < g.ny - 1 || g.bc[3] != BC_NOSLIP) &&
+         (z > 0 || g.bc[4] != BC_NOSLIP) && (z < g.nz - 1 || g.bc[5] != BC_NOSLIP);
 }
 // fast rows that touch no y or z face
 __device__ __forceinline__ bool interior_row(const Geom& g, int y, int z) {
-  return y > 0 && y < g.ny - 1 && z > 0 && z < g.nz - 1 && g.bc[0] != BC_NOSLIP && g.bc[1] != BC_NOSLIP;
+  return y > 0 && y < g.ny - 1 && z > 0 && z < g.nz - 1 && g.rows;
 }
 
 

@@ -66,6 +66,7 @@ def test_workspace_size_scales_with_storage(lib):
     dict(shape=(2, 8, 8)),
     dict(shape=(1200, 1200, 800)),                           # beyond the 2^30-node limit
     dict(shape=(6400, 6400, 3)),                             # xy plane beyond 32-bit slot offsets
+    dict(shape=(3, 10000, 6800)),                            # padded rows beyond 32-bit wraps in z
     dict(block=4),                                           # pipelined pass 1 outside compact storage
     dict(block=5),                                           # unknown block shape
     dict(bc=(5, 5, 0, 0, 0, 0)),                             # halo faces on x
