@@ -428,9 +428,9 @@ lbm_status lbm_create(int nx, int ny, int nz, const lbm_params* p, lbm** out) {
                                       : (packed ? 5 : 1));
   h->fix_ready = false;
   // block shape: as measured on GB300 (128x128x512 jet), the fused FP32 kernel runs fastest in
-  // 32x2x4 blocks (775 against 786 us a step for 32x4x2); every other kernel in 32x4x2
+  // 32x2x4 blocks (783 us a step against 793 for 32x4x2 and 819 for 32x8x1); every other kernel in 32x4x2
   h->shape = p->block != 0 ? p->block - 1 : (h->variant == 3 && p->storage == LBM_STORE_F32 ? 1 : 0);
-  // compact storage: the TMA-pipelined pass 1 wherever it applies (522 against 711 us a step on the jet)
+  // compact storage: the TMA-pipelined pass 1 wherever it applies (530 against 720 us a step on the jet)
   if (h->ks->compact && p->block == 0 && pipelined_ok(nx, ny, nz, p)) h->shape = 3;
   if (p->storage == LBM_STORE_F64) h->shape = 0;  // node after node, whatever was asked for
 

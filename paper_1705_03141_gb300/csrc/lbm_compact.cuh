@@ -68,7 +68,7 @@ struct CompactStore {
     }
     __stcs(A + e0 + dir * 32, float_to_dev(f - K.refB[cls]));
   }
-  // by a node's base pointer p1 = A + e1 and a 32-bit element offset (fast rows)
+  // by a node's base pointer p1 = A + e1 and an element offset (fast rows)
   __device__ __forceinline__ float load_rel(const uint16_t* p1, int64_t rel, int dir, int cls,
                                             const KConst<float>& K) const {
     if (dir == REST) {
@@ -300,8 +300,8 @@ __global__ void __launch_bounds__(NTHREADS, 3) k_density_c(CompactStore<BF16> st
 // by the producer lanes with 4-byte asynchronous copies that the stage's barrier also waits for.
 // At a reflecting x face the face lane reads plane p -/+ 2 of its own node instead (the mirror of
 // AoRow), and the record of the face node with m_x reversed (per-lane offsets and signs).
-// Coordinates outside the box read zeros.  Rows that are not fast rows (next to a y or z face, or
-// the outflow plane) are left out of the tiles, so no tile waits on global-memory latency: before
+// Coordinates outside the box read zeros.  Rows on a y or z face (the outflow plane among them) are
+// left out of the tiles, so no tile waits on global-memory latency: before
 // their first tile, all consumer warps of the grid share those rows, read from global memory
 // (dens_general), while the producers fill the first stages.  Periodic x faces keep the
 // one-block-per-tile kernel for the whole box.
@@ -469,7 +469,7 @@ __global__ void __launch_bounds__(NG * NTHREADS + 32, MINB)
     return;
   }
 
-  // first the rows that are not fast rows, shared among all consumer warps of the grid while the
+  // first the rows on y and z faces, shared among all consumer warps of the grid while the
   // producer fills the first stages: rows y = 0, ny - 1 (every z), then z = 0, nz - 1 (the y
   // between), in 32-node pieces
   {

@@ -346,7 +346,7 @@ inline RelaxConst<R> make_relax(const double rate[27]) {
 // there), which takes 488 instead of 515 us a step on the 128x128x512 jet; rounding once costs FP64
 // storage 3 % of a step (32^3 55.5 -> 57.2 us) and compact storage 1.5 % (128x128x512 536 -> 545 us).
 // Relaxing the 23 moments of Eq. (momentSet) one by one between T and T^-1, with the closed forms
-// added per raw moment, took about 330 operations.  Measured with the gradients by
+// added per raw moment, took about 330 operations.  Measured folded, with the gradients by
 // opposite pairs: collide-stream pass in FP64 on a 32^3 box (bound by the FP64 pipe) 69 -> 56 us;
 // packed half, interior tiles of a 128^3 jet 78 -> 72 us on even and 88 -> 85 us on odd steps.
 template <bool FOLD, typename R>
