@@ -952,27 +952,30 @@ lbm_status stage_inputs(lbm_mlp* m, const float* x, const float* target, const i
   return LBM_OK;
 }
 
-// may the kernels use the caller's buffer itself
-bool in_place(const lbm_mlp* m, const void* ptr) {
+// where a caller's buffer lies (one query each): on the host, on a device but to be staged, or where the
+// kernels use it themselves
+enum Place { ON_HOST, ON_DEVICE, IN_PLACE };
+Place place_of(const lbm_mlp* m, const void* ptr) {
   cudaPointerAttributes a;
-  if (!ptr) return false;
+  if (!ptr) return ON_HOST;
   if (cudaPointerGetAttributes(&a, ptr) != cudaSuccess) {
     cudaGetLastError();
-    return false;
+    return ON_HOST;
   }
-  return mlpbuf::in_place(a.type == cudaMemoryTypeDevice, a.type == cudaMemoryTypeManaged, a.device, m->device,
-                          reinterpret_cast<uintptr_t>(ptr));
+  const bool dev = a.type == cudaMemoryTypeDevice, managed = a.type == cudaMemoryTypeManaged;
+  if (mlpbuf::in_place(dev, managed, a.device, m->device, reinterpret_cast<uintptr_t>(ptr))) return IN_PLACE;
+  return dev || managed ? ON_DEVICE : ON_HOST;
 }
 
 // device pointer of an input: the caller's own where the kernels may use it and it stays as it is while
 // they run, else a copy at `staged`
 template <typename V>
-lbm_status on_device(lbm_mlp* m, const V* src, V* staged, size_t n, const V** out, bool stays = true) {
-  if (stays && in_place(m, src)) {
+lbm_status on_device(lbm_mlp* m, const V* src, Place at, V* staged, size_t n, const V** out, bool stays = true) {
+  if (stays && at == IN_PLACE) {
     *out = src;
     return LBM_OK;
   }
-  const cudaMemcpyKind k = is_device_ptr(src) ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
+  const cudaMemcpyKind k = at == ON_HOST ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice;
   MLP_CUDA(cudaMemcpyAsync(staged, src, sizeof(V) * n, k, m->stream));
   *out = staged;
   return LBM_OK;
@@ -986,7 +989,7 @@ lbm_status fused_forward(lbm_mlp* m, const float* x, int batch, float* y) {
   const size_t nx = (size_t)batch * m->n_in, ny = (size_t)batch * m->n_out;
   const bool apart = !mlpbuf::overlap(reinterpret_cast<uintptr_t>(x), sizeof(float) * nx,
                                       reinterpret_cast<uintptr_t>(y), sizeof(float) * ny);
-  lbm_status st = on_device(m, x, m->x32, nx, &A.x, apart);
+  lbm_status st = on_device(m, x, place_of(m, x), m->x32, nx, &A.x, apart);
   if (st != LBM_OK) return st;
   A.y = y;
   A.p = m->p;
@@ -1002,8 +1005,8 @@ lbm_status fused_backward(lbm_mlp* m, const float* x, const float* target, const
   RowsArgs A;
   memset(&A, 0, sizeof A);
   const size_t nx = (size_t)batch * m->n_in, nt = (size_t)batch * m->n_pos, nl = m->n_cls > 0 ? (size_t)batch : 0;
-  if (m->pinned && 4 * (nx + nt + nl) <= STAGE_BYTES && !is_device_ptr(x) && (!nt || !is_device_ptr(target)) &&
-      (!nl || !is_device_ptr(label))) {
+  const Place px = place_of(m, x), pt = nt ? place_of(m, target) : ON_HOST, pl = nl ? place_of(m, label) : ON_HOST;
+  if (m->pinned && 4 * (nx + nt + nl) <= STAGE_BYTES && px == ON_HOST && pt == ON_HOST && pl == ON_HOST) {
     // a small host batch: through page-locked memory in one copy (every call waits for its stream
     // before it returns, so the buffer is free again by the next)
     memcpy(m->pinned, x, 4 * nx);
@@ -1014,9 +1017,9 @@ lbm_status fused_backward(lbm_mlp* m, const float* x, const float* target, const
     A.target = A.x + nx;
     A.label = reinterpret_cast<const int*>(A.target + nt);
   } else {
-    lbm_status st = on_device(m, x, m->x32, nx, &A.x);
-    if (st == LBM_OK && nt) st = on_device(m, target, m->tgt, nt, &A.target);
-    if (st == LBM_OK && nl) st = on_device(m, label, m->lab, nl, &A.label);
+    lbm_status st = on_device(m, x, px, m->x32, nx, &A.x);
+    if (st == LBM_OK && nt) st = on_device(m, target, pt, m->tgt, nt, &A.target);
+    if (st == LBM_OK && nl) st = on_device(m, label, pl, m->lab, nl, &A.label);
     if (st != LBM_OK) return st;
   }
   WgradArgs G;
@@ -1250,7 +1253,7 @@ lbm_status lbm_mlp_forward(lbm_mlp* m, const float* x, int batch, float* y) {
   if (!m || !x || !y || batch < 1 || batch > m->max_batch) return LBM_EINVAL;
   lbm_status st;
   if (m->fused) {
-    const bool own = in_place(m, y);  // the answers go straight to the caller's device memory
+    const bool own = place_of(m, y) == IN_PLACE;  // the answers go straight to the caller's device memory
     st = fused_forward(m, x, batch, own ? y : m->y);
     if (st == LBM_OK && !own) st = copy_out(m, y, m->y, sizeof(float) * batch * m->n_out);
   } else {
