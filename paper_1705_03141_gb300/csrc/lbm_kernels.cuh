@@ -1545,12 +1545,13 @@ __global__ void __launch_bounds__(B::NT, MINB)
 // ---------------------------------------------------------------------------
 // FP64 storage: both passes node after node (thread n holds node n of the box, x fastest).  GB300
 // issues an FP64 instruction of a warp in 16 cycles whatever number of its lanes is active, and at
-// about 570 of them a node that is all the time there is (an SM's issue slots are 90 % idle).  So
+// about 610 of them a node that is all the time there is (an SM's issue slots are 90 % idle).  So
 // the lanes are filled first: rows of 41 nodes cost 41, not 64; small blocks spread a small box
 // over all SMs; and every node takes the general streaming map, which is integer work, so that a
 // warp may span rows.  The gradients read (rho, phi) through L1.
 // Against 32 x 4 x 2 blocks with a halo tile in shared memory, us a step: 32^3 58 -> 55, 41^3 168 ->
-// 105, 17x40x23 58 -> 33, 64^3 386 -> 354 (57, 109, 34 and 368 with the relaxation rounded once).
+// 105, 17x40x23 58 -> 33, 64^3 386 -> 354; 57, 109, 34 and 368 with the relaxation rounded once (19
+// cycles per FP64 instruction and SM of the pipe's 16).
 constexpr int LIN_THREADS = 64;
 
 __device__ __forceinline__ bool lin_node(const Geom& G, int& x, int& y, int& z) {
